@@ -307,9 +307,9 @@ rbt_status genp_update(int32_t prec, int64_t M, int64_t N, int64_t K, const floa
  * genp_solve -- B <- (L U)^{-1} B (trans = 0) or B <- (L U)^{-T} B
  * (trans = 1) with the factors of genp_factor (LU: n x n, lda, element type
  * per prec).  B: double, n x nrhs, ldb.  For float factors the solve runs in
- * float on a float copy of B held in `work` (genp_solve_workspace bytes) and
- * the result is widened back into B; for double-float factors (RBT_DF64,
- * RBT_DF64TC, RBT_DF64TC7) likewise in double-float arithmetic.  The first int of `work` is cleared on
+ * float (B rounded as it is read, the result widened back into B); for
+ * double-float factors (RBT_DF64, RBT_DF64TC, RBT_DF64TC7) likewise in
+ * double-float arithmetic.  work: genp_solve_workspace bytes.  The first int of `work` is cleared on
  * entry and is nonzero after a call whose chained triangular solve gave up
  * waiting (B is then undefined; see rbt_debug_wait_limit).
  */

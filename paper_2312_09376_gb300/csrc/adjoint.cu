@@ -201,19 +201,17 @@ rbt_status rbt_solve_adjoint(const rbt_opts *opts, const rbt_info *fwd, int64_t 
     double *R = (double *)(w + L.r);
     double *scal = (double *)(w + L.scal);  // [2] ||A^T||, [3] berr
     void *sol = w + L.sol;
-    size_t sol_bytes = L.total - L.sol;
     const int d = opts->depth;
     if (rbt_reference_size(n, d, opts->align, opts->grid_p, opts->grid_q) < 0) return RBT_ERR_ARG;
     const int64_t align = effective_align(opts->align, opts->grid_p, opts->grid_q);
-    auto corr = [&](double *Z, int64_t ldz) -> rbt_status {
+    auto corr = [&](double *Z, int64_t ldz, bool have_inv) -> rbt_status {
         // Z <- U A~^{-T} V^T Z
         rbt_status st = apply_vec(n, d, align, V, n, 1, Z, ldz, nrhs, s, opts->kind);
         if (st != RBT_OK) return st;
-        st = genp_solve_run(n, nrhs, prec, At, L.ldt, 1, Z, ldz, sol, s);
+        st = genp_solve_run(n, nrhs, prec, At, L.ldt, 1, Z, ldz, sol, have_inv, s);
         if (st != RBT_OK) return st;
         return apply_vec(n, d, align, U, n, 0, Z, ldz, nrhs, s, opts->kind);
     };
-    (void)sol_bytes;  // sized by the solve layout
     // the chained solves' timeout flag: cleared once, read before returning
     RBT_CUDA_TRY(cudaMemsetAsync(sol, 0, sizeof(int), s));
     auto timed_out = [&](bool *out) -> rbt_status {
@@ -224,7 +222,7 @@ rbt_status rbt_solve_adjoint(const rbt_opts *opts, const rbt_info *fwd, int64_t 
         return RBT_OK;
     };
     RBT_CUDA_TRY(cudaMemcpy2DAsync(Y, ldy * 8, G, ldg * 8, n * 8, nrhs, cudaMemcpyDeviceToDevice, s));
-    rbt_status st = corr(Y, ldy);
+    rbt_status st = corr(Y, ldy, false);
     if (st != RBT_OK) return st;
     st = resid_t(n, nrhs, A, lda, Y, ldy, G, ldg, R, n, scal + 2, true, scal + 3, s);
     if (st != RBT_OK) return st;
@@ -234,7 +232,7 @@ rbt_status rbt_solve_adjoint(const rbt_opts *opts, const rbt_info *fwd, int64_t 
     info->berr_unrefined = berr;
     int it = 0;
     while (!(berr <= opts->tol) && it < opts->refine_max) {
-        st = corr(R, n);
+        st = corr(R, n, true);
         if (st != RBT_OK) return st;
         st = add_block(n, nrhs, R, n, Y, ldy, s);
         if (st != RBT_OK) return st;

@@ -155,9 +155,7 @@ void solve_layout(const rbt_opts *o, int64_t n, int64_t nrhs, SolveLayout *out)
     L.scal = take(4 * 8);
     L.res = take(residual_ws(n, nr));
     L.fac = take(genp_factor_workspace_impl(n, o->prec, o->nb));
-    size_t sol_ws = genp_solve_workspace(n, nr, o->prec) + genp_solve_workspace(n, nr, RBT_F32);
-    if (o->refine_mode == RBT_REFINE_GMRES) sol_ws = std::max(sol_ws, genp_solve_wp_workspace(n, 1));
-    L.sol = take(sol_ws);
+    L.sol = take(genp_solve_workspace(n, nr, RBT_F64));  // 8-byte entries: covers every precision and the GMRES form
     if (o->refine_mode == RBT_REFINE_GMRES) {
         // basis Q (m + 1 columns), z, w, a zero vector, dot-product partials, h / y
         const int64_t m = o->restart > 0 ? o->restart : kGmresDefaultRestart;
@@ -204,13 +202,12 @@ rbt_status read_pivot_status(int64_t k, int prec, const void *At, int64_t ldt, c
 
 // dX = V A~^{-1} U^T R, in place in R
 rbt_status correction(int64_t n, int64_t nrhs, int d, int64_t align, int kind, const double *U, const double *V, int prec,
-                      const void *At, int64_t ldt, double *R, int64_t ldr, void *sol, size_t sol_bytes,
+                      const void *At, int64_t ldt, double *R, int64_t ldr, void *sol, bool have_inv,
                       cudaStream_t s)
 {
     rbt_status st = apply_vec(n, d, align, U, n, 1, R, ldr, nrhs, s, kind);
     if (st != RBT_OK) return st;
-    (void)sol_bytes;  // sized by the solve layout
-    st = genp_solve_run(n, nrhs, prec, At, ldt, 0, R, ldr, sol, s);
+    st = genp_solve_run(n, nrhs, prec, At, ldt, 0, R, ldr, sol, have_inv, s);
     if (st != RBT_OK) return st;
     return apply_vec(n, d, align, V, n, 0, R, ldr, nrhs, s, kind);
 }
@@ -219,12 +216,11 @@ rbt_status correction(int64_t n, int64_t nrhs, int d, int64_t align, int kind, c
 // factors: the preconditioner M^{-1} of GMRES-based refinement, applied in
 // the working precision so that it is the same linear operator every time.
 rbt_status precondition_wp(int64_t n, int d, int64_t align, int kind, const double *U, const double *V, int prec,
-                           const void *At, int64_t ldt, double *z, void *sol, size_t sol_bytes, cudaStream_t s)
+                           const void *At, int64_t ldt, double *z, void *sol, bool have_inv, cudaStream_t s)
 {
     rbt_status st = apply_vec(n, d, align, U, n, 1, z, n, 1, s, kind);
     if (st != RBT_OK) return st;
-    (void)sol_bytes;  // sized by the solve layout
-    st = genp_solve_wp_run(n, 1, prec, At, ldt, 0, z, n, sol, s);
+    st = genp_solve_wp_run(n, 1, prec, At, ldt, 0, z, n, sol, have_inv, s);
     if (st != RBT_OK) return st;
     return apply_vec(n, d, align, V, n, 0, z, n, 1, s, kind);
 }
@@ -233,8 +229,9 @@ rbt_status precondition_wp(int64_t n, int d, int64_t align, int kind, const doub
 // of at most m steps on A M^{-1} u = r with M^{-1} = V A~^{-1} U^T, the
 // Arnoldi vectors orthogonalized by classical Gram-Schmidt applied twice,
 // then x += M^{-1} Q y.  Adds the preconditioned products used to *used.
+// have_inv: sol holds the inverses of an earlier cycle with these factors.
 rbt_status gmres_cycle(int64_t n, int d, int64_t align, int kind, const double *U, const double *V, int prec, const void *At,
-                       int64_t ldt, void *sol, size_t sol_bytes, const double *A, int64_t lda,
+                       int64_t ldt, void *sol, bool have_inv, const double *A, int64_t lda,
                        const double *d_anorm, double *res_part, const double *r, double *x, int m, char *gw,
                        cudaStream_t s, int *used)
 {
@@ -265,7 +262,7 @@ rbt_status gmres_cycle(int64_t n, int d, int64_t align, int kind, const double *
     for (int j = 0; j < m; j++) {
         // w = A M^{-1} q_j
         RBT_CUDA_TRY(cudaMemcpyAsync(z, Q + (size_t)j * n, sizeof(double) * n, cudaMemcpyDeviceToDevice, s));
-        st = precondition_wp(n, d, align, kind, U, V, prec, At, ldt, z, sol, sol_bytes, s);
+        st = precondition_wp(n, d, align, kind, U, V, prec, At, ldt, z, sol, have_inv || j > 0, s);
         if (st != RBT_OK) return st;
         st = residual_impl(n, 1, A, lda, z, n, zero, n, w, n, d_anorm, dscr, res_part, s);  // w = -A z
         if (st != RBT_OK) return st;
@@ -317,7 +314,7 @@ rbt_status gmres_cycle(int64_t n, int d, int64_t align, int kind, const double *
     RBT_CUDA_TRY(cudaMemcpyAsync(dh, y.data(), sizeof(double) * k, cudaMemcpyHostToDevice, s));
     st = gm_gemv(n, Q, n, k, dh, z, s);
     if (st != RBT_OK) return st;
-    st = precondition_wp(n, d, align, kind, U, V, prec, At, ldt, z, sol, sol_bytes, s);
+    st = precondition_wp(n, d, align, kind, U, V, prec, At, ldt, z, sol, true, s);
     if (st != RBT_OK) return st;
     st = gm_add(n, z, x, s);
     if (st != RBT_OK) return st;
@@ -406,7 +403,7 @@ rbt_status rbt_solve(const rbt_opts *opts, int64_t n, int64_t nrhs, const double
     double *res = (double *)(w + L.res);
     void *fac = w + L.fac;
     void *sol = w + L.sol;
-    size_t fac_bytes = L.sol - L.fac, sol_bytes = L.total - L.sol;
+    size_t fac_bytes = L.sol - L.fac;
     const int64_t ldt = L.ldt;
     rbt_status st;
 
@@ -429,7 +426,7 @@ rbt_status rbt_solve(const rbt_opts *opts, int64_t n, int64_t nrhs, const double
 
     // 3. x = V A~^{-1} U^T b (steps 1-3), residual and backward error
     RBT_CUDA_TRY(cudaMemcpy2DAsync(X, ldx * 8, B, ldb * 8, n * 8, nrhs, cudaMemcpyDeviceToDevice, s));
-    st = correction(n, nrhs, d, align, opts->kind, U, V, prec, At, ldt, X, ldx, sol, sol_bytes, s);
+    st = correction(n, nrhs, d, align, opts->kind, U, V, prec, At, ldt, X, ldx, sol, false, s);
     if (st != RBT_OK) return st;
     st = residual_impl(n, nrhs, A, lda, X, ldx, B, ldb, R, n, scal, scal + 1, res, s);
     if (st != RBT_OK) return st;
@@ -460,6 +457,10 @@ rbt_status rbt_solve(const rbt_opts *opts, int64_t n, int64_t nrhs, const double
     }
     info->berr_unrefined = berr;
 
+    // whose diagonal-block inverses of the current factors sol holds: 0 =
+    // nobody's, 1 = the corrections', 2 = the GMRES preconditioner's
+    int inv_in_sol = 1;
+
     // 4. iterative refinement (Sec. 5); a stalled or exhausted low-precision
     //    attempt re-solves with a double factorization of the same A~
     int iters = 0, attempt_iters = 0, gm_products = 0;
@@ -487,6 +488,7 @@ rbt_status rbt_solve(const rbt_opts *opts, int64_t n, int64_t nrhs, const double
             cur_ldt = ldt;
             attempt_iters = 0;
             prev = INFINITY;
+            inv_in_sol = 1;  // by the correction below
             if (h_info >= 0) {
                 if (next != RBT_F64) {
                     berr = INFINITY;  // a failed factor counts as a stall: on to double
@@ -502,7 +504,7 @@ rbt_status rbt_solve(const rbt_opts *opts, int64_t n, int64_t nrhs, const double
                 return ps;
             }
             RBT_CUDA_TRY(cudaMemcpy2DAsync(X, ldx * 8, B, ldb * 8, n * 8, nrhs, cudaMemcpyDeviceToDevice, s));
-            st = correction(n, nrhs, d, align, opts->kind, U, V, cur_prec, cur_At, cur_ldt, X, ldx, sol, sol_bytes, s);
+            st = correction(n, nrhs, d, align, opts->kind, U, V, cur_prec, cur_At, cur_ldt, X, ldx, sol, false, s);
             if (st != RBT_OK) return st;
             st = residual_impl(n, nrhs, A, lda, X, ldx, B, ldb, R, n, scal, scal + 1, res, s);
             if (st != RBT_OK) return st;
@@ -514,13 +516,14 @@ rbt_status rbt_solve(const rbt_opts *opts, int64_t n, int64_t nrhs, const double
             const int m = opts->restart > 0 ? opts->restart : kGmresDefaultRestart;
             int used = 0;
             for (int64_t c = 0; c < nrhs; c++) {
-                st = gmres_cycle(n, d, align, opts->kind, U, V, cur_prec, cur_At, cur_ldt, sol, sol_bytes, A, lda, scal, res,
-                                 R + c * n, X + c * ldx, m, w + L.gm, s, &used);
+                st = gmres_cycle(n, d, align, opts->kind, U, V, cur_prec, cur_At, cur_ldt, sol, inv_in_sol == 2, A, lda, scal,
+                                 res, R + c * n, X + c * ldx, m, w + L.gm, s, &used);
                 if (st != RBT_OK) return st;
+                inv_in_sol = used > 0 ? 2 : 0;  // a cycle that took no product left sol as it was: compute anew
             }
             gm_products += used;
         } else {
-            st = correction(n, nrhs, d, align, opts->kind, U, V, cur_prec, cur_At, cur_ldt, R, n, sol, sol_bytes, s);
+            st = correction(n, nrhs, d, align, opts->kind, U, V, cur_prec, cur_At, cur_ldt, R, n, sol, inv_in_sol == 1, s);
             if (st != RBT_OK) return st;
             st = add_block(n, nrhs, R, n, X, ldx, s);
             if (st != RBT_OK) return st;

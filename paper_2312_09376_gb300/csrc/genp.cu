@@ -1,4 +1,5 @@
-// Gaussian elimination with no pivoting and its triangular solves (sm_103a).
+// Gaussian elimination with no pivoting (sm_103a); its triangular solves are in
+// trsv.cu.
 //
 // Blocked right-looking LU without row exchanges (Sec. 1; the GENP step of
 // Eq. precond).  Without pivoting the diagonal block needs nothing from the
@@ -605,851 +606,6 @@ rbt_status genp_configure(int prec, int nb)
     return configure_smem<float>(kMaxNB);
 }
 
-// ------------------------------------------------------- triangular solves
-
-// Diagonal block solve for every right-hand side: one CTA per column.
-// lower: unit lower L11 (trans 0) or U11^T (trans 1, non-unit);
-// upper: U11 (trans 0) or L11^T (trans 1, unit).
-template <typename T>
-__global__ void __launch_bounds__(128) trsv_diag_kernel(int64_t k0, int kb, const T *LU, int64_t lda, T *B,
-                                                        int64_t ldb, int lower, int trans)
-{
-    __shared__ T x[kMaxNB];
-    extern __shared__ unsigned char smem_raw[];
-    T *M = reinterpret_cast<T *>(smem_raw);  // kb x kb block of LU
-    const int tid = threadIdx.x;
-    const int64_t c = blockIdx.x;
-    for (int e = tid; e < kb * kb; e += blockDim.x) {
-        int i = e % kb, j = e / kb;
-        M[e] = LU[(k0 + i) + (k0 + j) * lda];
-    }
-    for (int i = tid; i < kb; i += blockDim.x) x[i] = B[(k0 + i) + c * ldb];
-    __syncthreads();
-    // op(M)(i, p): entry of the triangular matrix actually solved with
-    const bool unit = (lower && !trans) || (!lower && trans);
-    if (lower) {
-        for (int i = 0; i < kb; i++) {
-            if (tid == 0) {
-                T xi = x[i];
-                if (!unit) xi /= M[i + i * kb];
-                x[i] = xi;
-            }
-            __syncthreads();
-            T xi = x[i];
-            for (int r = i + 1 + tid; r < kb; r += blockDim.x) {
-                T m = trans ? M[i + r * kb] : M[r + i * kb];
-                x[r] -= m * xi;
-            }
-            __syncthreads();
-        }
-    } else {
-        for (int i = kb - 1; i >= 0; i--) {
-            if (tid == 0) {
-                T xi = x[i];
-                if (!unit) xi /= M[i + i * kb];
-                x[i] = xi;
-            }
-            __syncthreads();
-            T xi = x[i];
-            for (int r = tid; r < i; r += blockDim.x) {
-                T m = trans ? M[i + r * kb] : M[r + i * kb];
-                x[r] -= m * xi;
-            }
-            __syncthreads();
-        }
-    }
-    for (int i = tid; i < kb; i += blockDim.x) B[(k0 + i) + c * ldb] = x[i];
-}
-
-// y[rows] -= op(M)[rows, blk] * x[blk] for all rhs, notrans: M(r, p) = LU[r + p lda].
-// One thread per row; coalesced over rows.
-template <typename T>
-__global__ void __launch_bounds__(128) trsv_update_n_kernel(int64_t r0, int64_t r1, int64_t p0, int kb,
-                                                            const T *LU, int64_t lda, T *B, int64_t ldb,
-                                                            int64_t nrhs)
-{
-    __shared__ T xs[kMaxNB * 8];
-    const int64_t r = r0 + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    for (int64_t c0 = 0; c0 < nrhs; c0 += 8) {
-        int nc = (int)(nrhs - c0 < 8 ? nrhs - c0 : 8);
-        __syncthreads();
-        for (int e = threadIdx.x; e < kb * nc; e += blockDim.x) {
-            int p = e % kb, c = e / kb;
-            xs[c * kMaxNB + p] = B[(p0 + p) + (c0 + c) * ldb];
-        }
-        __syncthreads();
-        if (r < r1) {
-            T acc[8];
-#pragma unroll
-            for (int c = 0; c < 8; c++) acc[c] = T(0);
-            for (int p = 0; p < kb; p++) {
-                T m = LU[r + (p0 + p) * lda];
-#pragma unroll
-                for (int c = 0; c < 8; c++)
-                    if (c < nc) acc[c] = fma(m, xs[c * kMaxNB + p], acc[c]);
-            }
-            for (int c = 0; c < nc; c++) B[r + (c0 + c) * ldb] -= acc[c];
-        }
-    }
-}
-
-// transposed: M(r, p) = LU[p + r lda]; one warp per row, lanes over p.
-template <typename T>
-__global__ void __launch_bounds__(128) trsv_update_t_kernel(int64_t r0, int64_t r1, int64_t p0, int kb,
-                                                            const T *LU, int64_t lda, T *B, int64_t ldb,
-                                                            int64_t nrhs)
-{
-    const int lane = threadIdx.x & 31;
-    const int64_t r = r0 + ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32;
-    if (r >= r1) return;
-    for (int64_t c = 0; c < nrhs; c++) {
-        T acc = T(0);
-        for (int p = lane; p < kb; p += 32) acc = fma(LU[(p0 + p) + r * lda], B[(p0 + p) + c * ldb], acc);
-        for (int o = 16; o > 0; o >>= 1) acc += shfl_xor(acc, o);
-        if (lane == 0) B[r + c * ldb] -= acc;
-    }
-}
-
-template <typename T>
-static rbt_status tri_solve(int64_t n, int64_t nrhs, const T *LU, int64_t lda, int lower, int trans, T *B,
-                            int64_t ldb, int nb, cudaStream_t stream)
-{
-    const int64_t nblk = cdiv(n, nb);
-    for (int64_t bi = 0; bi < nblk; bi++) {
-        int64_t blk = lower ? bi : (nblk - 1 - bi);
-        int64_t k0 = blk * nb;
-        int kb = (int)(n - k0 < nb ? n - k0 : nb);
-        for (int64_t c0 = 0; c0 < nrhs; c0 += 65535) {
-            int64_t nc = nrhs - c0 < 65535 ? nrhs - c0 : 65535;
-            trsv_diag_kernel<T><<<(unsigned)nc, 128, (size_t)kb * kb * sizeof(T), stream>>>(
-                k0, kb, LU, lda, B + c0 * ldb, ldb, lower, trans);
-            RBT_LAUNCH_CHECK();
-        }
-        int64_t r0 = lower ? k0 + kb : 0, r1 = lower ? n : k0;
-        if (r1 <= r0) continue;
-        if (!trans) {
-            trsv_update_n_kernel<T><<<(unsigned)cdiv(r1 - r0, 128), 128, 0, stream>>>(r0, r1, k0, kb, LU, lda, B,
-                                                                                       ldb, nrhs);
-        } else {
-            trsv_update_t_kernel<T><<<(unsigned)cdiv((r1 - r0) * 32, 128), 128, 0, stream>>>(r0, r1, k0, kb, LU,
-                                                                                              lda, B, ldb, nrhs);
-        }
-        RBT_LAUNCH_CHECK();
-    }
-    return RBT_OK;
-}
-
-// ------------------------------------------- chained triangular solve
-
-// One persistent launch per triangle.  Row blocks of kChainNB rows are taken
-// in solve order from a device counter; the CTA holding block b streams the
-// columns of all earlier blocks that are already finished (four column lanes
-// per row, many loads in flight; warp 0 finds the finished prefix 32 flags at
-// a time), and when it has caught up it fetches its entries of the next
-// block's columns before waiting for that block's solution.  It then finishes
-// its diagonal block with the precomputed inverse plus one correction step
-// (x0 = D^-1 r, x = x0 + D^-1 (r - D x0), each product split over the four
-// lanes) and publishes it.  A CTA only waits on blocks taken before its own, which belong
-// to running CTAs, so the chain always advances; every wait is bounded and
-// records a timeout in err instead of hanging.
-//
-// The time per block on the chain is what the solve costs (the streaming
-// keeps up easily): the wait for the previous block's flag, then its columns,
-// the lane reduction and the three block products.  So the kernel is compiled
-// for the number R of right-hand sides it carries per pass (one, the common
-// case, or kChainRhs), its block's right-hand side is read before the wait,
-// and every per-lane sum runs as two interleaved chains (even and odd column
-// groups, fixed by the column index so the rounding does not depend on how
-// the finished columns were grouped).
-constexpr int kChainNB = 64;
-constexpr int kChainLanes = 4;                          // column lanes per row when streaming
-constexpr int kChainThreads = kChainNB * kChainLanes;  // 256
-constexpr int kChainRhs = 8;                            // right-hand sides per pass beyond one
-
-// An entry of the stored factor in the solve's arithmetic type T: the same
-// type, a float widened to double, or a double-float pair rounded to double.
-template <typename T, typename TF> __device__ __forceinline__ T elem_as(TF v) { return T(v); }
-template <> __device__ __forceinline__ double elem_as<double, df64>(df64 v) { return df_to_double(v); }
-
-// Inverse of every diagonal block of the triangle op(M) solves with (lower or
-// upper part of LU or of LU^T, unit diagonal where the factor has one): one
-// CTA per block, thread c computes column c of the inverse by substitution.
-// The chained solve then finishes a block with a parallel product instead of
-// a serial substitution on its critical path.
-template <typename T, typename TF = T>
-__global__ void __launch_bounds__(kChainNB) diag_inv_kernel(int64_t n, const TF *__restrict__ LU, int64_t lda,
-                                                            int lower, int trans, T *inv)
-{
-    __shared__ T D[kChainNB][kChainNB + 1];
-    __shared__ T X[kChainNB][kChainNB + 1];
-    const int c = threadIdx.x;
-    const int64_t pb = blockIdx.x;
-    const int64_t r0 = pb * kChainNB;
-    const int kb = (int)(n - r0 < kChainNB ? n - r0 : kChainNB);
-    const bool unit = (lower && !trans) || (!lower && trans);
-    for (int e = c; e < kChainNB * kChainNB; e += kChainNB) {
-        int r = trans ? e / kChainNB : e % kChainNB, p = trans ? e % kChainNB : e / kChainNB;
-        D[r][p] = (r < kb && p < kb) ? elem_as<T>(trans ? LU[(r0 + p) + (r0 + r) * lda] : LU[(r0 + r) + (r0 + p) * lda])
-                                     : T(0);
-    }
-    __syncthreads();
-    if (c < kb) {
-        if (lower) {
-            for (int i = 0; i < kb; i++) {
-                if (i < c) {
-                    X[i][c] = T(0);
-                    continue;
-                }
-                T s = (i == c) ? T(1) : T(0);
-                for (int p = c; p < i; p++) s -= D[i][p] * X[p][c];
-                X[i][c] = unit ? s : s / D[i][i];
-            }
-        } else {
-            for (int i = kb - 1; i >= 0; i--) {
-                if (i > c) {
-                    X[i][c] = T(0);
-                    continue;
-                }
-                T s = (i == c) ? T(1) : T(0);
-                for (int p = i + 1; p <= c; p++) s -= D[i][p] * X[p][c];
-                X[i][c] = unit ? s : s / D[i][i];
-            }
-        }
-    }
-    __syncthreads();
-    T *out = inv + pb * kChainNB * kChainNB;  // column-major 64 x 64, zero outside kb x kb
-    for (int e = c; e < kChainNB * kChainNB; e += kChainNB) {
-        int r = e % kChainNB, q = e / kChainNB;
-        out[e] = (r < kb && q < kb) ? X[r][q] : T(0);
-    }
-}
-
-template <typename T, typename TF, int R>
-__global__ void __launch_bounds__(kChainThreads, R == 1 ? 2 : 1)
-trsv_chain_kernel(int64_t n, int64_t nrhs, const TF *__restrict__ LU, int64_t lda, int lower, int trans, T *X,
-                  int64_t ldx, int *flags, int *counter, int *err, const T *__restrict__ inv, int first_blk,
-                  long long wait_ns)
-{
-    // dynamic shared memory (T):
-    //   D[64][65]      diagonal block of op(M)
-    //   Di[64][65]     its inverse (from diag_inv_kernel)
-    //   xs[64][R+1]    right-hand sides of the block, R columns per pass
-    //   red[4][64][R]  partial sums of the four column lanes
-    extern __shared__ __align__(16) unsigned char chain_smem[];
-    typedef T Row[kChainNB + 1];
-    typedef T RowS[R + 1];
-    Row *D = reinterpret_cast<Row *>(chain_smem);
-    Row *Di = D + kChainNB;
-    RowS *xs = reinterpret_cast<RowS *>(Di + kChainNB);
-    T *red = reinterpret_cast<T *>(xs + kChainNB);
-    __shared__ int s_blk, s_hi;
-    constexpr int U = kChainNB / kChainLanes;  // columns of one block per lane
-    const int tid = threadIdx.x;
-    const int rr = tid % kChainNB, pl = tid / kChainNB;  // row of the block, column lane
-    const int64_t nblk = (n + kChainNB - 1) / kChainNB;
-    // physical block of solve step j, and the columns [cb, ce) of steps j0 .. j1-1
-    auto phys = [&](int64_t j) { return lower ? j : nblk - 1 - j; };
-    auto col_range = [&](int64_t j0, int64_t j1, int64_t &cb, int64_t &ce) {
-        cb = lower ? j0 * kChainNB : (nblk - j1) * kChainNB;
-        ce = lower ? j1 * kChainNB : (nblk - j0) * kChainNB;
-        if (ce > n) ce = n;
-    };
-    for (;;) {
-        if (tid == 0) s_blk = first_blk + atomicAdd(counter, 1);
-        __syncthreads();
-        const int64_t b = s_blk;
-        __syncthreads();
-        if (b >= nblk) return;
-        const int64_t pb = phys(b);
-        const int64_t r0 = pb * kChainNB;
-        const int kb = (int)(n - r0 < kChainNB ? n - r0 : kChainNB);
-        const bool unit = (lower && !trans) || (!lower && trans);
-        for (int e = tid; e < kChainNB * kChainNB; e += kChainThreads) {
-            // only the triangle being solved with, unit diagonal where the factor has one
-            const int r = trans ? e / kChainNB : e % kChainNB, p = trans ? e % kChainNB : e / kChainNB;
-            const bool in_tri = r < kb && p < kb && (lower ? p <= r : p >= r);
-            T v = T(0);
-            if (in_tri)
-                v = (p == r && unit) ? T(1)
-                                     : elem_as<T>(trans ? LU[(r0 + p) + (r0 + r) * lda] : LU[(r0 + r) + (r0 + p) * lda]);
-            D[r][p] = v;
-            Di[e % kChainNB][e / kChainNB] = inv[pb * kChainNB * kChainNB + e];
-        }
-        const int64_t grow = r0 + rr;
-        auto entry = [&](int64_t p) { return elem_as<T>(trans ? LU[p + grow * lda] : LU[grow + p * lda]); };
-        for (int64_t c0 = 0; c0 < nrhs; c0 += R) {
-            const int nc = R == 1 ? 1 : (int)(nrhs - c0 < R ? nrhs - c0 : R);
-            // the block's own right-hand sides stay as they are until it is solved
-            T rhs[R];
-#pragma unroll
-            for (int c = 0; c < R; c++) rhs[c] = (pl == 0 && rr < kb && c < nc) ? X[grow + (c0 + c) * ldx] : T(0);
-            T acc0[R], acc1[R];
-#pragma unroll
-            for (int c = 0; c < R; c++) acc0[c] = acc1[c] = T(0);
-            // column p = cb + pl + 4 q of this lane: q's parity picks the chain
-            // (cb is a multiple of 64, so the parity is that of p / 4)
-            auto mac = [&](T(&acc)[R], T m, int64_t p) {
-#pragma unroll
-                for (int c = 0; c < R; c++)
-                    if (c < nc) acc[c] = fma(m, ld_cg(X + p + (c0 + c) * ldx), acc[c]);
-            };
-            for (int64_t jl = 0; jl < b;) {
-                // finished prefix [jl, hi) of the earlier steps: warp 0 reads 32 flags per round
-                if (tid < 32) {
-                    int64_t hi = jl;
-                    for (;;) {
-                        const int64_t q = hi + tid;
-                        const bool rdy = q < b && *((volatile int *)(flags + phys(q))) != 0;
-                        const unsigned m = __ballot_sync(0xffffffffu, rdy);
-                        if (m == 0xffffffffu) {
-                            hi += 32;
-                            if (hi < b) continue;
-                            hi = b;
-                        } else {
-                            hi += __ffs(~m) - 1;
-                        }
-                        break;
-                    }
-                    __threadfence();
-                    if (tid == 0) s_hi = (int)hi;
-                }
-                __syncthreads();
-                const int64_t hi = s_hi;
-                int64_t cb, ce;
-                if (hi > jl) {
-                    col_range(jl, hi, cb, ce);
-                    // A lower solve meets its finished steps in ascending column
-                    // order and an upper one in descending order, whatever the
-                    // grouping of the steps into chunks, when each chunk is walked
-                    // the same way: so each chain's summation order (and the
-                    // rounding) is the same on every run.
-                    const int64_t span = ce - cb - pl;
-                    if (rr < kb && span > 0) {
-                        const int64_t qn = (span - 1) / kChainLanes + 1;
-                        auto col = [&](int64_t q) { return cb + pl + kChainLanes * q; };
-                        if (lower) {
-                            int64_t q = 0;
-#pragma unroll 2
-                            for (; q + 1 < qn; q += 2) {
-                                const T m0 = entry(col(q)), m1 = entry(col(q + 1));
-                                mac(acc0, m0, col(q));
-                                mac(acc1, m1, col(q + 1));
-                            }
-                            if (q < qn) mac(acc0, entry(col(q)), col(q));
-                        } else {
-                            int64_t q = qn - 1;
-                            if (q & 1) {
-                                mac(acc1, entry(col(q)), col(q));
-                                q--;
-                            }
-#pragma unroll 2
-                            for (; q >= 1; q -= 2) {
-                                const T m0 = entry(col(q)), m1 = entry(col(q - 1));
-                                mac(acc0, m0, col(q));
-                                mac(acc1, m1, col(q - 1));
-                            }
-                            if (q == 0) mac(acc0, entry(col(0)), col(0));
-                        }
-                    }
-                    jl = hi;
-                } else {
-                    // step jl is the front and not finished: its entries in this row
-                    // block are final already, so fetch them before waiting
-                    col_range(jl, jl + 1, cb, ce);
-                    T mp[U];
-#pragma unroll
-                    for (int u = 0; u < U; u++) {
-                        const int64_t p = cb + pl + kChainLanes * u;
-                        mp[u] = (rr < kb && p < ce) ? entry(p) : T(0);
-                    }
-                    if (tid == 0) {
-                        // bounded by wait_ns of %globaltimer; a timeout (or one
-                        // seen from another CTA) ends every later wait at once
-                        const int64_t pj = phys(jl);
-                        unsigned long long t0 = 0;
-                        bool timing = false;
-                        while (*((volatile int *)(flags + pj)) == 0 && *((volatile int *)err) == 0) {
-                            if (!timing) {
-                                t0 = global_ns();
-                                timing = true;
-                            } else if ((long long)(global_ns() - t0) > wait_ns) {
-                                atomicExch(err, 1);
-                                break;
-                            }
-                            __nanosleep(32);
-                        }
-                        __threadfence();
-                    }
-                    __syncthreads();
-                    if (rr < kb) {
-                        // the same per-lane column order and chains as the chunked form
-                        auto step_u = [&](int u) {
-                            const int64_t p = cb + pl + kChainLanes * u;
-                            if (p < ce) {
-                                if (u & 1)
-                                    mac(acc1, mp[u], p);
-                                else
-                                    mac(acc0, mp[u], p);
-                            }
-                        };
-                        if (lower) {
-#pragma unroll
-                            for (int u = 0; u < U; u++) step_u(u);
-                        } else {
-#pragma unroll
-                            for (int u = U - 1; u >= 0; u--) step_u(u);
-                        }
-                    }
-                    jl += 1;
-                }
-                __syncthreads();
-            }
-            // reduce the column lanes; residual right-hand side of the block
-#pragma unroll
-            for (int c = 0; c < R; c++) red[(pl * kChainNB + rr) * R + c] = acc0[c] + acc1[c];
-            __syncthreads();
-            auto lane_sum = [&](int c) {
-                T s = red[rr * R + c];
-                for (int l = 1; l < kChainLanes; l++) s += red[(l * kChainNB + rr) * R + c];
-                return s;
-            };
-            if (pl == 0 && rr < kb) {
-#pragma unroll
-                for (int c = 0; c < R; c++)
-                    if (c < nc) {
-                        rhs[c] -= lane_sum(c);
-                        xs[rr][c] = rhs[c];
-                    }
-            }
-            __syncthreads();
-            // block solve D x = r: x0 = Di r, then one correction x = x0 + Di (r - D x0).
-            // Each product is split over the four column lanes (16 terms each,
-            // two chains) and summed through shared memory; row rr's lane 0
-            // keeps r and x0 in registers.  Each row's lane 0 only rewrites its
-            // own row of xs, after the barrier that ends the product reading it.
-            auto lane_products = [&](const Row *Mx) {
-                T q0[R], q1[R];
-#pragma unroll
-                for (int c = 0; c < R; c++) q0[c] = q1[c] = T(0);
-                if (rr < kb) {
-#pragma unroll
-                    for (int u = 0; u < U; u++) {
-                        const int p = pl + kChainLanes * u;
-                        if (p < kb) {
-                            const T m = Mx[rr][p];
-#pragma unroll
-                            for (int c = 0; c < R; c++)
-                                if (c < nc) {
-                                    if (u & 1)
-                                        q1[c] = fma(m, xs[p][c], q1[c]);
-                                    else
-                                        q0[c] = fma(m, xs[p][c], q0[c]);
-                                }
-                        }
-                    }
-                }
-#pragma unroll
-                for (int c = 0; c < R; c++) red[(pl * kChainNB + rr) * R + c] = q0[c] + q1[c];
-            };
-            T x0[R];
-            lane_products(Di);  // x0 = Di r
-            __syncthreads();
-            if (pl == 0 && rr < kb) {
-#pragma unroll
-                for (int c = 0; c < R; c++)
-                    if (c < nc) {
-                        x0[c] = lane_sum(c);
-                        xs[rr][c] = x0[c];
-                    }
-            }
-            __syncthreads();
-            lane_products(D);  // D x0
-            __syncthreads();
-            if (pl == 0 && rr < kb) {
-#pragma unroll
-                for (int c = 0; c < R; c++)
-                    if (c < nc) xs[rr][c] = rhs[c] - lane_sum(c);
-            }
-            __syncthreads();
-            lane_products(Di);  // Di (r - D x0)
-            __syncthreads();
-            if (pl == 0 && rr < kb) {
-#pragma unroll
-                for (int c = 0; c < R; c++)
-                    if (c < nc) X[grow + (c0 + c) * ldx] = x0[c] + lane_sum(c);
-            }
-            if (R > 1) __syncthreads();  // xs and red are reused by the next pass
-        }
-        __threadfence();
-        __syncthreads();
-        if (tid == 0) atomicExch(flags + pb, 1);
-    }
-}
-
-template <typename T, int R> constexpr size_t chain_smem_bytes()
-{
-    return (2 * kChainNB * (kChainNB + 1) + kChainNB * (R + 1) + kChainLanes * kChainNB * R) * sizeof(T);
-}
-
-template <typename T, typename TF, int R>
-static rbt_status launch_chain(int64_t n, int64_t nrhs, const TF *LU, int64_t lda, int lower, int trans, T *B,
-                               int64_t ldb, int *scratch, const T *inv, cudaStream_t stream)
-{
-    static PerDeviceOnce once;
-    rbt_status cst = smem_opt_in(once, trsv_chain_kernel<T, TF, R>, (int)chain_smem_bytes<T, R>());
-    if (cst != RBT_OK) return cst;
-    const int64_t nblk = cdiv(n, kChainNB);
-    int *err = scratch, *counter = scratch + 1, *flags = scratch + 2;
-    RBT_CUDA_TRY(cudaMemsetAsync(counter, 0, sizeof(int) * (size_t)(nblk + 1), stream));
-    int per_sm = 1;
-    RBT_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, trsv_chain_kernel<T, TF, R>, kChainThreads,
-                                                               chain_smem_bytes<T, R>()));
-    int64_t grid = (int64_t)device_sm_count() * (per_sm > 0 ? per_sm : 1);
-    if (grid > nblk) grid = nblk;
-    // the test stall starts the queue at block 1: block 0 is never solved
-    const int first_blk = debug_stall() == RBT_STALL_CHAIN ? 1 : 0;
-    trsv_chain_kernel<T, TF, R><<<(unsigned)grid, kChainThreads, chain_smem_bytes<T, R>(), stream>>>(
-        n, nrhs, LU, lda, lower, trans, B, ldb, flags, counter, err, inv, first_blk, wait_limit_ns());
-    RBT_LAUNCH_CHECK();
-    return RBT_OK;
-}
-
-// scratch: [0] timeout flag (cleared by the public entry point or the solve
-// driver, once per call: it stays set across the triangles and refinement
-// steps of one call), [1] block counter, [2..] block flags, then (256-byte
-// aligned) the inverses of the diagonal blocks.
-template <typename T, typename TF = T>
-static rbt_status tri_chain(int64_t n, int64_t nrhs, const TF *LU, int64_t lda, int lower, int trans, T *B,
-                            int64_t ldb, int *scratch, cudaStream_t stream)
-{
-    const int64_t nblk = cdiv(n, kChainNB);
-    T *inv = (T *)((char *)scratch + ((size_t)(nblk + 2) * sizeof(int) + 255) / 256 * 256);
-    diag_inv_kernel<T, TF><<<(unsigned)nblk, kChainNB, 0, stream>>>(n, LU, lda, lower, trans, inv);
-    RBT_LAUNCH_CHECK();
-    if (nrhs == 1) return launch_chain<T, TF, 1>(n, nrhs, LU, lda, lower, trans, B, ldb, scratch, inv, stream);
-    return launch_chain<T, TF, kChainRhs>(n, nrhs, LU, lda, lower, trans, B, ldb, scratch, inv, stream);
-}
-
-size_t chain_scratch_bytes(int64_t n, size_t es)
-{
-    const int64_t nblk = cdiv(n > 0 ? n : 1, kChainNB);
-    return ((size_t)(nblk + 2) * sizeof(int) + 255) / 256 * 256 + (size_t)nblk * kChainNB * kChainNB * es + 256;
-}
-
-// ------------------------------------- blocked solves for many right-hand sides
-//
-// With many right-hand sides the chain's per-block critical path grows with
-// them (a block is published only after all its right-hand sides); a
-// right-looking blocked solve is then faster: for each 64-row block in solve
-// order, finish the block with its precomputed inverse plus one correction
-// step, then subtract its contribution from all the rows still to solve with
-// one wide update kernel.
-constexpr int kBlkRhs = 32;       // right-hand sides per pass of the block kernels
-constexpr int kBlkRhsMin = 4;     // fewer right-hand sides take the chained solve
-
-// X_b <- op(M)_bb^{-1} X_b for step block pb: x0 = Di r, x = x0 + Di (r - D x0).
-template <typename T>
-__global__ void __launch_bounds__(256) blk_diag_kernel(int64_t n, int64_t nrhs, const T *__restrict__ LU,
-                                                       int64_t lda, int lower, int trans, int64_t pb,
-                                                       const T *__restrict__ inv, T *X, int64_t ldx)
-{
-    extern __shared__ __align__(16) unsigned char blk_smem[];
-    typedef T Row[kChainNB + 1];
-    typedef T RowR[kBlkRhs + 1];
-    Row *D = reinterpret_cast<Row *>(blk_smem);
-    Row *Di = D + kChainNB;
-    RowR *r = reinterpret_cast<RowR *>(Di + kChainNB);
-    RowR *x0 = r + kChainNB;
-    const int tid = threadIdx.x;
-    const int64_t r0 = pb * kChainNB;
-    const int kb = (int)(n - r0 < kChainNB ? n - r0 : kChainNB);
-    const bool unit = (lower && !trans) || (!lower && trans);
-    for (int e = tid; e < kChainNB * kChainNB; e += 256) {
-        const int i = trans ? e / kChainNB : e % kChainNB, p = trans ? e % kChainNB : e / kChainNB;
-        const bool in_tri = i < kb && p < kb && (lower ? p <= i : p >= i);
-        T v = T(0);
-        if (in_tri) v = (p == i && unit) ? T(1) : (trans ? LU[(r0 + p) + (r0 + i) * lda] : LU[(r0 + i) + (r0 + p) * lda]);
-        D[i][p] = v;
-        Di[e % kChainNB][e / kChainNB] = inv[pb * kChainNB * kChainNB + e];
-    }
-    for (int64_t c0 = 0; c0 < nrhs; c0 += kBlkRhs) {
-        const int nc = (int)(nrhs - c0 < kBlkRhs ? nrhs - c0 : kBlkRhs);
-        for (int e = tid; e < kChainNB * kBlkRhs; e += 256) {
-            const int i = e % kChainNB, c = e / kChainNB;
-            r[i][c] = (i < kb && c < nc) ? X[(r0 + i) + (c0 + c) * ldx] : T(0);
-        }
-        __syncthreads();
-        // x0 = Di r
-        for (int e = tid; e < kChainNB * kBlkRhs; e += 256) {
-            const int i = e % kChainNB, c = e / kChainNB;
-            T s = T(0);
-            for (int p = 0; p < kb; p++) s = fma(Di[i][p], r[p][c], s);
-            x0[i][c] = s;
-        }
-        __syncthreads();
-        // r <- r - D x0 (each entry read and written by its own thread)
-        for (int e = tid; e < kChainNB * kBlkRhs; e += 256) {
-            const int i = e % kChainNB, c = e / kChainNB;
-            T s = r[i][c];
-            for (int p = 0; p < kb; p++) s -= D[i][p] * x0[p][c];
-            r[i][c] = s;
-        }
-        __syncthreads();
-        // x = x0 + Di r
-        for (int e = tid; e < kChainNB * kBlkRhs; e += 256) {
-            const int i = e % kChainNB, c = e / kChainNB;
-            if (i < kb && c < nc) {
-                T s = x0[i][c];
-                for (int p = 0; p < kb; p++) s = fma(Di[i][p], r[p][c], s);
-                X[(r0 + i) + (c0 + c) * ldx] = s;
-            }
-        }
-        __syncthreads();
-    }
-}
-
-// C (M x N) -= A (M x K) Xb (K x N), K <= 64, for the rows still to solve:
-// A column-major (lda), or its transpose when TA (A(i, k) at A[k + i lda]).
-// One row per thread, Xb staged in shared memory kBlkRhs columns at a time.
-template <typename T, bool TA>
-__global__ void __launch_bounds__(128) blk_update_kernel(int64_t M, int64_t N, int K, const T *__restrict__ A,
-                                                         int64_t lda, const T *Xb, int64_t ldx, T *C, int64_t ldc)
-{
-    __shared__ T xs[kChainNB][kBlkRhs + 1];
-    const int64_t i = (int64_t)blockIdx.x * 128 + threadIdx.x;
-    for (int64_t c0 = 0; c0 < N; c0 += kBlkRhs) {
-        const int nc = (int)(N - c0 < kBlkRhs ? N - c0 : kBlkRhs);
-        for (int e = threadIdx.x; e < kChainNB * kBlkRhs; e += 128) {
-            const int k = e % kChainNB, c = e / kChainNB;
-            xs[k][c] = (k < K && c < nc) ? Xb[k + (c0 + c) * ldx] : T(0);
-        }
-        __syncthreads();
-        if (i < M) {
-            T acc[kBlkRhs];
-#pragma unroll
-            for (int c = 0; c < kBlkRhs; c++) acc[c] = T(0);
-            for (int k = 0; k < K; k++) {
-                const T a = TA ? A[k + i * lda] : A[i + (int64_t)k * lda];
-#pragma unroll
-                for (int c = 0; c < kBlkRhs; c++) acc[c] = fma(a, xs[k][c], acc[c]);
-            }
-#pragma unroll
-            for (int c = 0; c < kBlkRhs; c++)
-                if (c < nc) C[i + (c0 + c) * ldc] -= acc[c];
-        }
-        __syncthreads();
-    }
-}
-
-template <typename T> constexpr size_t blk_diag_smem_bytes()
-{
-    return (2 * kChainNB * (kChainNB + 1) + 2 * kChainNB * (kBlkRhs + 1)) * sizeof(T);
-}
-
-// One triangle of op(M) (as tri_chain) by blocks; the inverses of the
-// diagonal blocks go to the chain scratch's inverse area.
-template <typename T>
-static rbt_status tri_blocked(int64_t n, int64_t nrhs, const T *LU, int64_t lda, int lower, int trans, T *B,
-                              int64_t ldb, int *scratch, cudaStream_t stream)
-{
-    const int64_t nblk = cdiv(n, kChainNB);
-    T *inv = (T *)((char *)scratch + ((size_t)(nblk + 2) * sizeof(int) + 255) / 256 * 256);
-    diag_inv_kernel<T><<<(unsigned)nblk, kChainNB, 0, stream>>>(n, LU, lda, lower, trans, inv);
-    RBT_LAUNCH_CHECK();
-    static PerDeviceOnce once;
-    rbt_status cst = smem_opt_in(once, blk_diag_kernel<T>, (int)blk_diag_smem_bytes<T>());
-    if (cst != RBT_OK) return cst;
-    for (int64_t j = 0; j < nblk; j++) {
-        const int64_t pb = lower ? j : nblk - 1 - j;
-        const int64_t r0 = pb * kChainNB;
-        const int kb = (int)(n - r0 < kChainNB ? n - r0 : kChainNB);
-        blk_diag_kernel<T><<<1, 256, blk_diag_smem_bytes<T>(), stream>>>(n, nrhs, LU, lda, lower, trans, pb, inv, B,
-                                                                         ldb);
-        RBT_LAUNCH_CHECK();
-        // rows still to solve: below the block (lower) or above it (upper)
-        const int64_t m0 = lower ? r0 + kb : 0, M = lower ? n - r0 - kb : r0;
-        if (M <= 0) continue;
-        // op(M)(m0 + i, r0 + k): the lower part is L (trans = 0) or U^T (trans = 1),
-        // the upper part U (trans = 0) or L^T (trans = 1)
-        const unsigned grid = (unsigned)cdiv(M, 128);
-        if (!trans) {
-            blk_update_kernel<T, false><<<grid, 128, 0, stream>>>(M, nrhs, kb, LU + m0 + r0 * lda, lda, B + r0, ldb,
-                                                                  B + m0, ldb);
-        } else {
-            blk_update_kernel<T, true><<<grid, 128, 0, stream>>>(M, nrhs, kb, LU + r0 + m0 * lda, lda, B + r0, ldb,
-                                                                 B + m0, ldb);
-        }
-        RBT_LAUNCH_CHECK();
-    }
-    return RBT_OK;
-}
-
-// (L U)^{-1} B or (L U)^{-T} B: two chained launches, or two blocked sweeps
-// for many right-hand sides; scratch[0] (device) becomes nonzero when a wait
-// of the chained form gave up, and is never cleared here.
-template <typename T>
-rbt_status lu_solve_chain(int64_t n, int64_t nrhs, const T *LU, int64_t lda, int trans, T *B, int64_t ldb,
-                          int *scratch, cudaStream_t stream)
-{
-    ProfScope ps(kProfSolve, stream);
-    if (nrhs >= kBlkRhsMin) {
-        rbt_status st = tri_blocked<T>(n, nrhs, LU, lda, 1, trans, B, ldb, scratch, stream);
-        if (st != RBT_OK) return st;
-        return tri_blocked<T>(n, nrhs, LU, lda, 0, trans, B, ldb, scratch, stream);
-    }
-    rbt_status st = tri_chain<T>(n, nrhs, LU, lda, 1, trans, B, ldb, scratch, stream);  // L y = b or U^T y = b
-    if (st != RBT_OK) return st;
-    return tri_chain<T>(n, nrhs, LU, lda, 0, trans, B, ldb, scratch, stream);           // U x = y or L^T x = y
-}
-
-// (L U)^{-1} B or (L U)^{-T} B in double arithmetic with factors stored in a
-// lower precision TF (float, or double-float pairs): the chained form, any
-// number of right-hand sides.  Each entry is widened as it is read, so the
-// solve reads the factors' own bytes and the only error beyond the factors'
-// is that of a double substitution.
-template <typename TF>
-static rbt_status lu_solve_wp(int64_t n, int64_t nrhs, const TF *LU, int64_t lda, int trans, double *B, int64_t ldb,
-                              int *scratch, cudaStream_t stream)
-{
-    ProfScope ps(kProfSolve, stream);
-    rbt_status st = tri_chain<double, TF>(n, nrhs, LU, lda, 1, trans, B, ldb, scratch, stream);
-    if (st != RBT_OK) return st;
-    return tri_chain<double, TF>(n, nrhs, LU, lda, 0, trans, B, ldb, scratch, stream);
-}
-
-template <typename T>
-rbt_status lu_solve(int64_t n, int64_t nrhs, const T *LU, int64_t lda, int trans, T *B, int64_t ldb,
-                    cudaStream_t stream)
-{
-    ProfScope ps(kProfSolve, stream);
-    static PerDeviceOnce once;
-    rbt_status cst = smem_opt_in(once, trsv_diag_kernel<T>, (int)(kSolveNB * kSolveNB * sizeof(T)));
-    if (cst != RBT_OK) return cst;
-    rbt_status st;
-    if (!trans) {
-        st = tri_solve<T>(n, nrhs, LU, lda, 1, 0, B, ldb, kSolveNB, stream);  // L y = b
-        if (st != RBT_OK) return st;
-        return tri_solve<T>(n, nrhs, LU, lda, 0, 0, B, ldb, kSolveNB, stream);  // U x = y
-    }
-    st = tri_solve<T>(n, nrhs, LU, lda, 1, 1, B, ldb, kSolveNB, stream);  // U^T y = b
-    if (st != RBT_OK) return st;
-    return tri_solve<T>(n, nrhs, LU, lda, 0, 1, B, ldb, kSolveNB, stream);  // L^T x = y
-}
-
-template rbt_status lu_solve<double>(int64_t, int64_t, const double *, int64_t, int, double *, int64_t,
-                                     cudaStream_t);
-template rbt_status lu_solve<float>(int64_t, int64_t, const float *, int64_t, int, float *, int64_t, cudaStream_t);
-template rbt_status lu_solve<df64>(int64_t, int64_t, const df64 *, int64_t, int, df64 *, int64_t, cudaStream_t);
-
-// -------------------------------------------------------- conversions
-
-__global__ void narrow_kernel(int64_t n, int64_t nrhs, const double *B, int64_t ldb, float *F, int64_t ldf)
-{
-    int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (idx >= n * nrhs) return;
-    int64_t i = idx % n, c = idx / n;
-    F[i + c * ldf] = (float)B[i + c * ldb];
-}
-
-__global__ void widen_kernel(int64_t n, int64_t nrhs, const float *F, int64_t ldf, double *B, int64_t ldb)
-{
-    int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (idx >= n * nrhs) return;
-    int64_t i = idx % n, c = idx / n;
-    B[i + c * ldb] = (double)F[i + c * ldf];
-}
-
-__global__ void narrow_df_kernel(int64_t n, int64_t nrhs, const double *B, int64_t ldb, df64 *F, int64_t ldf)
-{
-    int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (idx >= n * nrhs) return;
-    int64_t i = idx % n, c = idx / n;
-    F[i + c * ldf] = df_from_double(B[i + c * ldb]);
-}
-
-__global__ void widen_df_kernel(int64_t n, int64_t nrhs, const df64 *F, int64_t ldf, double *B, int64_t ldb)
-{
-    int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (idx >= n * nrhs) return;
-    int64_t i = idx % n, c = idx / n;
-    B[i + c * ldb] = df_to_double(F[i + c * ldf]);
-}
-
-rbt_status narrow_block(int64_t n, int64_t nrhs, const double *B, int64_t ldb, float *F, int64_t ldf,
-                        cudaStream_t stream)
-{
-    if (n * nrhs == 0) return RBT_OK;
-    narrow_kernel<<<(unsigned)cdiv(n * nrhs, 256), 256, 0, stream>>>(n, nrhs, B, ldb, F, ldf);
-    RBT_LAUNCH_CHECK();
-    return RBT_OK;
-}
-
-rbt_status widen_block(int64_t n, int64_t nrhs, const float *F, int64_t ldf, double *B, int64_t ldb,
-                       cudaStream_t stream)
-{
-    if (n * nrhs == 0) return RBT_OK;
-    widen_kernel<<<(unsigned)cdiv(n * nrhs, 256), 256, 0, stream>>>(n, nrhs, F, ldf, B, ldb);
-    RBT_LAUNCH_CHECK();
-    return RBT_OK;
-}
-
-static rbt_status narrow_block_df(int64_t n, int64_t nrhs, const double *B, int64_t ldb, df64 *F, int64_t ldf,
-                                  cudaStream_t stream)
-{
-    if (n * nrhs == 0) return RBT_OK;
-    narrow_df_kernel<<<(unsigned)cdiv(n * nrhs, 256), 256, 0, stream>>>(n, nrhs, B, ldb, F, ldf);
-    RBT_LAUNCH_CHECK();
-    return RBT_OK;
-}
-
-static rbt_status widen_block_df(int64_t n, int64_t nrhs, const df64 *F, int64_t ldf, double *B, int64_t ldb,
-                                 cudaStream_t stream)
-{
-    if (n * nrhs == 0) return RBT_OK;
-    widen_df_kernel<<<(unsigned)cdiv(n * nrhs, 256), 256, 0, stream>>>(n, nrhs, F, ldf, B, ldb);
-    RBT_LAUNCH_CHECK();
-    return RBT_OK;
-}
-
-// genp_solve / genp_solve_wp after validation, without clearing the timeout
-// flag at the front of work (the caller owns its lifetime).
-rbt_status genp_solve_run(int64_t n, int64_t nrhs, int32_t prec, const void *LU, int64_t lda, int32_t trans,
-                          double *B, int64_t ldb, void *work, cudaStream_t stream)
-{
-    if (n == 0 || nrhs == 0) return RBT_OK;
-    int *scratch = (int *)work;
-    const size_t wes = prec == RBT_F64 ? sizeof(double) : ((is_df64_storage(prec)) ? sizeof(df64) : sizeof(float));
-    char *rest = (char *)work + ((chain_scratch_bytes(n, wes) + 255) / 256 * 256);
-    if (prec == RBT_F64)
-        return lu_solve_chain<double>(n, nrhs, (const double *)LU, lda, trans ? 1 : 0, B, ldb, scratch, stream);
-    if (is_df64_storage(prec)) {
-        df64 *F = (df64 *)rest;
-        rbt_status st = narrow_block_df(n, nrhs, B, ldb, F, n, stream);
-        if (st != RBT_OK) return st;
-        st = lu_solve_chain<df64>(n, nrhs, (const df64 *)LU, lda, trans ? 1 : 0, F, n, scratch, stream);
-        if (st != RBT_OK) return st;
-        return widen_block_df(n, nrhs, F, n, B, ldb, stream);
-    }
-    float *F = (float *)rest;
-    rbt_status st = narrow_block(n, nrhs, B, ldb, F, n, stream);
-    if (st != RBT_OK) return st;
-    st = lu_solve_chain<float>(n, nrhs, (const float *)LU, lda, trans ? 1 : 0, F, n, scratch, stream);
-    if (st != RBT_OK) return st;
-    return widen_block(n, nrhs, F, n, B, ldb, stream);
-}
-
-rbt_status genp_solve_wp_run(int64_t n, int64_t nrhs, int32_t prec, const void *LU, int64_t lda, int32_t trans,
-                             double *B, int64_t ldb, void *work, cudaStream_t stream)
-{
-    if (n == 0 || nrhs == 0) return RBT_OK;
-    int *scratch = (int *)work;
-    const int t = trans ? 1 : 0;
-    if (prec == RBT_F64) return lu_solve_chain<double>(n, nrhs, (const double *)LU, lda, t, B, ldb, scratch, stream);
-    if (is_df64_storage(prec))
-        return lu_solve_wp<df64>(n, nrhs, (const df64 *)LU, lda, t, B, ldb, scratch, stream);
-    return lu_solve_wp<float>(n, nrhs, (const float *)LU, lda, t, B, ldb, scratch, stream);
-}
-
 }  // namespace rbt
 
 using namespace rbt;
@@ -1471,48 +627,6 @@ rbt_status genp_factor(int64_t n, int32_t prec, void *A, int64_t lda, int64_t *d
     if (!A) return RBT_ERR_ARG;
     if (work_bytes < genp_factor_workspace_impl(n, prec, nb)) return RBT_ERR_WORKSPACE;
     return genp_factor_impl(n, prec, A, lda, d_info, work, work_bytes, nb, stream);
-}
-
-size_t genp_solve_workspace(int64_t n, int64_t nrhs, int32_t prec)
-{
-    if (n <= 0 || nrhs <= 0) return 0;
-    size_t es = prec == RBT_F64 ? 0 : ((is_df64_storage(prec)) ? sizeof(df64) : sizeof(float));
-    size_t ws = prec == RBT_F64 ? sizeof(double) : (es ? es : sizeof(float));
-    return (size_t)n * (size_t)nrhs * es + chain_scratch_bytes(n, ws) + 256;
-}
-
-// Solve flag at the front of the workspace: nonzero after a call whose chained
-// triangular solve gave up waiting (the result is then undefined).  The public
-// calls clear it on entry; the *_run forms (the solve driver's) never clear it,
-// so that one timeout stays visible for the rest of the driver's call.
-rbt_status genp_solve(int64_t n, int64_t nrhs, int32_t prec, const void *LU, int64_t lda, int32_t trans,
-                      double *B, int64_t ldb, void *work, size_t work_bytes, cudaStream_t stream)
-{
-    if (n < 0 || nrhs < 0 || prec < RBT_F64 || prec > kLastPrec) return RBT_ERR_ARG;
-    if (lda < (n > 1 ? n : 1) || ldb < (n > 1 ? n : 1)) return RBT_ERR_ARG;
-    if (n == 0 || nrhs == 0) return RBT_OK;
-    if (!LU || !B) return RBT_ERR_ARG;
-    if (work_bytes < genp_solve_workspace(n, nrhs, prec) || !work) return RBT_ERR_WORKSPACE;
-    RBT_CUDA_TRY(cudaMemsetAsync(work, 0, sizeof(int), stream));
-    return genp_solve_run(n, nrhs, prec, LU, lda, trans, B, ldb, work, stream);
-}
-
-size_t genp_solve_wp_workspace(int64_t n, int64_t nrhs)
-{
-    if (n <= 0 || nrhs <= 0) return 0;
-    return chain_scratch_bytes(n, sizeof(double)) + 256;
-}
-
-rbt_status genp_solve_wp(int64_t n, int64_t nrhs, int32_t prec, const void *LU, int64_t lda, int32_t trans,
-                         double *B, int64_t ldb, void *work, size_t work_bytes, cudaStream_t stream)
-{
-    if (n < 0 || nrhs < 0 || prec < RBT_F64 || prec > kLastPrec) return RBT_ERR_ARG;
-    if (lda < (n > 1 ? n : 1) || ldb < (n > 1 ? n : 1)) return RBT_ERR_ARG;
-    if (n == 0 || nrhs == 0) return RBT_OK;
-    if (!LU || !B) return RBT_ERR_ARG;
-    if (work_bytes < genp_solve_wp_workspace(n, nrhs) || !work) return RBT_ERR_WORKSPACE;
-    RBT_CUDA_TRY(cudaMemsetAsync(work, 0, sizeof(int), stream));
-    return genp_solve_wp_run(n, nrhs, prec, LU, lda, trans, B, ldb, work, stream);
 }
 
 }  // extern "C"

@@ -9,7 +9,6 @@ namespace rbt {
 constexpr int kMaxNB = 128;       // largest GENP block size (shared-memory bound)
 constexpr int kDefaultNB64 = 64;  // default block size, double
 constexpr int kDefaultNB32 = 128; // default block size, float storage
-constexpr int kSolveNB = 128;     // block size of the triangular solves
 
 // C (M x N) -= A (M x K) B (K x N), SIMT, column-major.
 template <typename T>
@@ -23,15 +22,6 @@ rbt_status genp_panel_steps(int64_t n, T *A, int64_t lda, int64_t *info, int nb,
                             bool trailing_simt, cudaStream_t stream);
 
 rbt_status genp_configure(int prec, int nb);
-
-template <typename T>
-rbt_status lu_solve(int64_t n, int64_t nrhs, const T *LU, int64_t lda, int trans, T *B, int64_t ldb,
-                    cudaStream_t stream);
-
-rbt_status narrow_block(int64_t n, int64_t nrhs, const double *B, int64_t ldb, float *F, int64_t ldf,
-                        cudaStream_t stream);
-rbt_status widen_block(int64_t n, int64_t nrhs, const float *F, int64_t ldf, double *B, int64_t ldb,
-                       cudaStream_t stream);
 
 size_t residual_ws(int64_t n, int64_t nrhs);
 // bytes of the partial sums residual_impl / norm_inf_impl write into `part`
@@ -75,10 +65,12 @@ rbt_status gm_add(int64_t n, const double *z, double *x, cudaStream_t s);
 // genp_solve / genp_solve_wp on validated arguments (work of their size
 // queries), leaving the timeout flag at the front of work as it is: set by a
 // chained solve that gave up, cleared only by whoever owns the call.
+// have_inv: work still holds the diagonal blocks' inverses that the same
+// function left there for the same factors, precision, orientation and nrhs.
 rbt_status genp_solve_run(int64_t n, int64_t nrhs, int32_t prec, const void *LU, int64_t lda, int32_t trans,
-                          double *B, int64_t ldb, void *work, cudaStream_t stream);
+                          double *B, int64_t ldb, void *work, bool have_inv, cudaStream_t stream);
 rbt_status genp_solve_wp_run(int64_t n, int64_t nrhs, int32_t prec, const void *LU, int64_t lda, int32_t trans,
-                             double *B, int64_t ldb, void *work, cudaStream_t stream);
+                             double *B, int64_t ldb, void *work, bool have_inv, cudaStream_t stream);
 
 size_t genp_factor_workspace_impl(int64_t n, int prec, int nb);
 rbt_status genp_factor_impl(int64_t n, int prec, void *A, int64_t lda, int64_t *info, void *work,
