@@ -471,10 +471,12 @@ def run_ours(args):
     del A_host, hwork
     torch.cuda.empty_cache()
 
-    # one FP64 solve of the same system (the comparison path), not part of the value
+    # one solve of the same system on the FP64 pipe (the comparison path: an
+    # explicit block size keeps the double updates off the tensor cores), not
+    # part of the value
     fp64 = None
     if not args.no_fp64 and rank == 0:
-        o64 = _lib.make_opts(depth=d, seed=1, prec="f64", refine_max=30, tol=1e-13, fallback=False)
+        o64 = _lib.make_opts(depth=d, seed=1, prec="f64", refine_max=30, tol=1e-13, fallback=False, nb=64)
         w64 = torch.empty(_lib.rbt_solve_workspace(o64, n, 1), dtype=torch.uint8, device=dev)
         h0 = torch.cuda.Event(enable_timing=True)
         h1 = torch.cuda.Event(enable_timing=True)

@@ -60,7 +60,12 @@ typedef enum {
 
 /* Working precision of the factorization. */
 typedef enum {
-    RBT_F64 = 0,   /* double storage and arithmetic */
+    RBT_F64 = 0,   /* double storage and arithmetic; rbt_solve with nb = 0 and
+                      n >= 1024 runs the factorization's updates by exact digit
+                      slicing on the BF16 tensor cores (nine 7-bit digits, 63
+                      bits relative to each row's and column's largest entry)
+                      when A~ is dense enough for that to be no less accurate
+                      than double multiply-adds */
     RBT_F32 = 1,   /* float storage, float SIMT trailing updates */
     RBT_TF32 = 2,  /* float storage, TF32 tensor-core trailing updates (fp32 accumulate) */
     RBT_BF16 = 3,  /* float storage, BF16 tensor-core operands (fp32 accumulate) */

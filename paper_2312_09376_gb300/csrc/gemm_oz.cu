@@ -29,6 +29,19 @@
 // same binade (on RBT-transformed GENP panels the bound relative to the
 // entrywise one drops from about 2^12 to 2^4 in the median).
 //
+// Double operands (RBT_F64, from n = 1024) take the same route with nine
+// digits: 63 bits relative to the row and column maxima, ten more than an
+// entry has, 45 products, K <= 448 (9 K 2^12 <= 2^24), 48-column tiles (nine
+// accumulators in TMEM), the fold in 64-bit integers.  Measured against the
+// FP64-pipe update (first backward errors of unrefined solves, n = 600 ..
+// 8197, depths 1 .. 3, both butterflies, rows and columns scaled by up to
+// 10^3: geometric mean of the ratio 0.3 .. 1.7 per family, 0.96 over all).
+// Entry by entry that holds where rows and columns are filled with entries of
+// like size; a sparse matrix's fill-in can be smaller than its row's maximum
+// by more than the ten spare bits, so rbt_solve asks first (spread.cu).  The
+// FP64 pipe's 1.2 TFLOP/s bounded such factorizations: update class at n =
+// 8197 307 ms, now 15.7 ms and 9.5 ms of slicing.
+//
 // Kernel: persistent, one CTA per SM, 128 x 64 output tiles (S accumulators
 // x 64 columns in the 512 TMEM columns) dealt round-robin in an L2-friendly
 // grouped order; a TMA producer warp streams 32-element K slabs of all S
@@ -45,6 +58,7 @@
 
 #include <algorithm>
 #include <mutex>
+#include <type_traits>
 
 #include "df64.cuh"
 #include "gemm_tc.cuh"
@@ -55,15 +69,17 @@ namespace oz {
 
 constexpr int BETA = 7;     // bits per digit
 constexpr int BM = 128;
-// TMEM holds one 128 x BN FP32 accumulator per digit weight t = 2 .. S + 1
-// (S accumulators, S <= 8) in 512 columns.
-constexpr int BN = 64;
+// TMEM holds one 128 x BN FP32 accumulator per digit weight t = 2 .. S + 1 in
+// 512 columns: 64 columns each for S = 7 and 8, 48 for S = 9.
+template <int S> constexpr int BN = S <= 8 ? 64 : 48;
+// digit slices of B that one MMA covers (N = 256, or 240 of 48-column slices)
+template <int S> constexpr int QN = 256 / BN<S>;
 constexpr int KSLAB = 32;   // bf16 elements per 64-byte row
 constexpr int A_SLICE_BYTES = BM * 64;
-constexpr int B_SLICE_BYTES = BN * 64;
-// S digits per operand (7 or 8): the stage ring is sized per digit count
-template <int S> constexpr int kStageBytes = S * (A_SLICE_BYTES + B_SLICE_BYTES);  // S = 8: 96 KB
-template <int S> constexpr int kStages = (227 * 1024 - 2048) / kStageBytes<S>;     // S = 7, 8: 2
+template <int S> constexpr int B_SLICE_BYTES = BN<S> * 64;
+// S digits per operand: the stage ring is sized per digit count
+template <int S> constexpr int kStageBytes = S * (A_SLICE_BYTES + B_SLICE_BYTES<S>);  // S = 8: 96 KB, 9: 99 KB
+template <int S> constexpr int kStages = (227 * 1024 - 2048) / kStageBytes<S>;        // 2
 template <int S> constexpr int kSmemBytes = kStages<S> * kStageBytes<S> + 1024 + 256;
 constexpr int kOzEpiWarps = 8;                    // epilogue warps (two per TMEM lane quarter)
 constexpr int kProdWarp = kOzEpiWarps;            // TMA producer
@@ -72,16 +88,25 @@ constexpr int kOzThreads = (kOzEpiWarps + 2) * 32;
 constexpr int TMEM_COLS = 512;
 // a digit product is at most 64 * 64 = 2^12 and a weight holds at most S of
 // them per k: S * K * 2^12 <= 2^24 keeps every accumulation exact
-constexpr int KMAX = 512;
-constexpr int kMaxDigits = 8;
-static_assert(kMaxDigits * KMAX * 4096 <= (1 << 24), "digit accumulation must stay exact");
-static_assert(kMaxDigits * BN <= TMEM_COLS, "one accumulator per digit weight in TMEM");
-static_assert(kStages<8> >= 2 && kStages<7> >= 2, "at least double buffering");
+template <int S> constexpr int KMAX = S <= 8 ? 512 : 448;
+constexpr int kMaxDigits = 8;    // of double-float operands
+constexpr int kDigits64 = 9;     // of double operands: 63 bits
+static_assert(kMaxDigits * KMAX<8> * 4096 <= (1 << 24) && kDigits64 * KMAX<9> * 4096 <= (1 << 24),
+              "digit accumulation must stay exact");
+static_assert(kMaxDigits * BN<8> <= TMEM_COLS && kDigits64 * BN<9> <= TMEM_COLS,
+              "one accumulator per digit weight in TMEM");
+static_assert(kStages<9> >= 2 && kStages<8> >= 2 && kStages<7> >= 2, "at least double buffering");
+// digits of an operand type's updates and back
+template <int S> using elem_t = std::conditional_t<S == kDigits64, double, df64>;
 constexpr int kGroupM = 16;  // row tiles per group of the tile order (L2 reuse of the digit slices)
 
 struct Status {
     int err;
 };
+
+// exponent of a row or column with an entry that is not finite (double
+// operands), above every exponent that occurs
+constexpr int kBadExp = 1 << 28;
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -160,6 +185,13 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32])
                  : "r"(taddr));
 }
 
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t *r)
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr));
+}
+
 // Wait for this thread's TMEM loads; the loaded registers are operands, so
 // that no use of them is scheduled before the wait.
 __device__ __forceinline__ void tmem_wait32(uint32_t (&r)[32])
@@ -172,6 +204,40 @@ __device__ __forceinline__ void tmem_wait32(uint32_t (&r)[32])
                    "+r"(r[29]), "+r"(r[30]), "+r"(r[31])
                  :
                  : "memory");
+}
+
+__device__ __forceinline__ void tmem_ld24(uint32_t taddr, uint32_t (&r)[24])
+{
+    tmem_ld8(taddr, r);
+    tmem_ld8(taddr + 8, r + 8);
+    tmem_ld8(taddr + 16, r + 16);
+}
+
+__device__ __forceinline__ void tmem_wait24(uint32_t (&r)[24])
+{
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                   "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]),
+                   "+r"(r[15]), "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]),
+                   "+r"(r[22]), "+r"(r[23])
+                 :
+                 : "memory");
+}
+
+// An integer of |v| < 2^51 as a double, in one FP64 addition (the conversion
+// instruction is no faster than that here, and an exact one in int32 is not
+// wide enough).
+__device__ __forceinline__ double double_of(long long v)
+{
+    return __longlong_as_double(0x4338000000000000ll + v) - 6755399441055744.0;  // 1.5 * 2^52
+}
+
+// C - v 2^e, v exact or rounded once; e outside the double exponents takes
+// the library's scaling.
+__device__ __forceinline__ double sub_scaled(double c, double v, int e)
+{
+    if (e > -1000 && e < 900) return ::fma(-v, __longlong_as_double((long long)(e + 1023) << 52), c);
+    return c - ldexp(v, e);
 }
 
 __device__ __forceinline__ float pow2f(int e)
@@ -204,7 +270,7 @@ __device__ __forceinline__ bool mbar_wait_ab(uint64_t *bar, uint32_t parity, Sta
 // inner within a group: the tiles in flight at one time share a band of
 // kGroupM x 128 rows of A's digit slices and a few column tiles of B's, both
 // L2-resident, instead of every wave streaming A's slices from DRAM.
-__device__ __forceinline__ void tile_origin(int64_t i, int tiles_m, int tiles_n, int &m0, int &n0)
+__device__ __forceinline__ void tile_origin(int64_t i, int tiles_m, int tiles_n, int bn, int &m0, int &n0)
 {
     const int64_t t = blockIdx.x + i * gridDim.x;
     const int64_t per_group = (int64_t)kGroupM * tiles_n;
@@ -212,7 +278,7 @@ __device__ __forceinline__ void tile_origin(int64_t i, int tiles_m, int tiles_n,
     const int first_m = grp * kGroupM;
     const int gm = tiles_m - first_m < kGroupM ? tiles_m - first_m : kGroupM;
     m0 = (first_m + in_grp % gm) * BM;
-    n0 = (in_grp / gm) * BN;
+    n0 = (in_grp / gm) * bn;
 }
 
 // C (df64, M x N, ldc) -= A B from the digit slices; ea[m] / fb[n] are the
@@ -242,7 +308,7 @@ template <bool RAW, int S>
 __global__ void __launch_bounds__(kOzThreads, 1)
 oz_update_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_b, int M,
                  int N, int K, int Mp, int Np, int a0, int b0, const int *__restrict__ ea, const int *__restrict__ fb,
-                 df64 *__restrict__ C, int64_t ldc, const int64_t *info, Status *st, long long wait_ns,
+                 elem_t<S> *__restrict__ C, int64_t ldc, const int64_t *info, Status *st, long long wait_ns,
                  int no_copy, float *__restrict__ raw)
 {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -255,10 +321,10 @@ oz_update_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
     uint32_t *tmem_slot = (uint32_t *)(drain + 1);
     volatile int *abort = (volatile int *)(tmem_slot + 1);
 
-    static_assert(S >= 5 && S <= kMaxDigits, "digit count");
+    static_assert(S >= 5 && S <= kDigits64, "digit count");
     if (*((volatile const int64_t *)info) >= 0) return;
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-    const int tiles_m = (M + BM - 1) / BM, tiles_n = (N + BN - 1) / BN;
+    const int tiles_m = (M + BM - 1) / BM, tiles_n = (N + BN<S> - 1) / BN<S>;
     const int64_t ntiles = (int64_t)tiles_m * tiles_n;
     if ((int64_t)blockIdx.x >= ntiles) return;
     const int64_t my_tiles = (ntiles - blockIdx.x + gridDim.x - 1) / gridDim.x;
@@ -292,7 +358,7 @@ oz_update_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
             int64_t g = 0;
             for (int64_t i = 0; i < my_tiles && !*abort && !no_copy; i++) {
                 int m0, n0;
-                tile_origin(i, tiles_m, tiles_n, m0, n0);
+                tile_origin(i, tiles_m, tiles_n, BN<S>, m0, n0);
                 for (int kt = 0; kt < nk; kt++, g++) {
                     const int s = (int)(g % kStages<S>);
                     const int64_t r = g / kStages<S>;
@@ -304,7 +370,7 @@ oz_update_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
                                  : "memory");
                     for (int p = 0; p < S; p++) {
                         tma_load_2d(sa + p * A_SLICE_BYTES, &tmap_a, kt * KSLAB, p * Mp + a0 + m0, &full[s]);
-                        tma_load_2d(sb + p * B_SLICE_BYTES, &tmap_b, kt * KSLAB, p * Np + b0 + n0, &full[s]);
+                        tma_load_2d(sb + p * B_SLICE_BYTES<S>, &tmap_b, kt * KSLAB, p * Np + b0 + n0, &full[s]);
                     }
                 }
             }
@@ -334,18 +400,18 @@ oz_update_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
                     // Digit p of A meets digits q = 1 .. S + 1 - p of B, whose
                     // accumulators (weights p + q) are adjacent in TMEM and whose
                     // slices are adjacent in shared memory: one MMA covers up to
-                    // four of them (N = 256).  p = 1 writes every accumulator first.
+                    // QN of them (N <= 256).  p = 1 writes every accumulator first.
 #pragma unroll
                     for (int p = 1; p <= S; p++) {
 #pragma unroll
-                        for (int q0 = 1; q0 <= S + 1 - p; q0 += 4) {
-                            const int nq = (S + 1 - p - q0 + 1) < 4 ? (S + 1 - p - q0 + 1) : 4;
-                            const uint32_t dcol = tmem + (uint32_t)((p + q0 - 2) * BN);
+                        for (int q0 = 1; q0 <= S + 1 - p; q0 += QN<S>) {
+                            const int nq = (S + 1 - p - q0 + 1) < QN<S> ? (S + 1 - p - q0 + 1) : QN<S>;
+                            const uint32_t dcol = tmem + (uint32_t)((p + q0 - 2) * BN<S>);
 #pragma unroll
                             for (int kk = 0; kk < 2; kk++) {
                                 const uint32_t acc = (kt > 0 || p > 1 || kk > 0) ? 1u : 0u;
                                 mma_bf16_n(dcol, smem_desc64(sa + (p - 1) * A_SLICE_BYTES + kk * 32),
-                                           smem_desc64(sb + (q0 - 1) * B_SLICE_BYTES + kk * 32), idesc_n(nq * BN),
+                                           smem_desc64(sb + (q0 - 1) * B_SLICE_BYTES<S> + kk * 32), idesc_n(nq * BN<S>),
                                            acc);
                             }
                         }
@@ -362,19 +428,19 @@ oz_update_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
         __syncwarp();
     } else {
         // epilogue warps
-        constexpr int EC = BN / 2;  // columns per warp
+        constexpr int EC = BN<S> / 2;  // columns per warp
         const int q = warp % 4, ch = warp / 4;  // TMEM lane quarter, half of the tile's columns
         const uint32_t lane_base = (uint32_t)(q * 32) << 16;
         for (int64_t i = 0; i < my_tiles; i++) {
             int m0, n0;
-            tile_origin(i, tiles_m, tiles_n, m0, n0);
+            tile_origin(i, tiles_m, tiles_n, BN<S>, m0, n0);
             const int row = m0 + q * 32 + lane;
             const bool rok = row < M;
             const int cbase = ch * EC;
-            // this tile's block of C towards L2 while its MMAs run: 64
+            // this tile's block of C towards L2 while its MMAs run: BN
             // columns, nine addresses each (one per 16 rows and the last row)
             if (!RAW)
-                for (int e = threadIdx.x; e < BN * 9; e += kOzEpiWarps * 32) {
+                for (int e = threadIdx.x; e < BN<S> * 9; e += kOzEpiWarps * 32) {
                     const int c = e / 9, r = e % 9;
                     const int gi = m0 + (r < 8 ? r * 16 : BM - 1), gj = n0 + c;
                     if (gi < M && gj < N) asm volatile("prefetch.global.L2 [%0];" ::"l"(C + gi + (int64_t)gj * ldc));
@@ -389,7 +455,7 @@ oz_update_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
 #pragma unroll 1
                 for (int t = 0; t < S; t++) {
                     uint32_t a[EC];
-                    tmem_ld32(base + (uint32_t)(t * BN), a);
+                    tmem_ld32(base + (uint32_t)(t * BN<S>), a);
                     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
                     if (rok)
                         for (int j = 0; j < EC; j++) {
@@ -402,6 +468,72 @@ oz_update_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
                 if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(tmem_empty)) : "memory");
                 continue;
             }
+            if constexpr (S == kDigits64) {
+                // Double.  The accumulators are integers, and the product is
+                // (H 2^28 + L) 2^(e_i + f_j - 70) with H = sum_{t <= 6} acc_t
+                // 2^(7 (6 - t)) and L = sum_{t >= 7} acc_t 2^(7 (10 - t)):
+                // gathered in 64-bit integers (neighbours first in 32 bits,
+                // within 2^31: at most (t - 1) K 2^12 each), |H| < 2^50 and
+                // |L| < 2^45 become doubles exactly.  Four FP64 operations an
+                // entry, after the accumulators are released: nine
+                // multiply-adds would take the FP64 pipe as long as the
+                // tile's MMAs take the tensor pipe.
+                long long H[EC], L[EC];
+                uint32_t r0[EC], r1[EC];
+                tmem_ld24(base, r0);
+                tmem_ld24(base + (uint32_t)BN<S>, r1);
+                tmem_wait24(r0);
+                tmem_wait24(r1);
+                auto both = [](uint32_t hi, uint32_t lo) {
+                    return __float2int_rn(__uint_as_float(hi)) * 128 + __float2int_rn(__uint_as_float(lo));
+                };
+#pragma unroll
+                for (int j = 0; j < EC; j++) H[j] = both(r0[j], r1[j]);                       // t = 2, 3
+                auto next = [&](int t, bool pair) {  // accumulators t and t + 1
+                    tmem_ld24(base + (uint32_t)((t - 2) * BN<S>), r0);
+                    if (pair) tmem_ld24(base + (uint32_t)((t - 1) * BN<S>), r1);
+                    tmem_wait24(r0);
+                    if (pair) tmem_wait24(r1);
+                };
+                next(4, true);
+#pragma unroll
+                for (int j = 0; j < EC; j++) H[j] = (H[j] << 14) + both(r0[j], r1[j]);        // 4, 5
+                next(6, false);
+#pragma unroll
+                for (int j = 0; j < EC; j++) H[j] = (H[j] << 7) + __float2int_rn(__uint_as_float(r0[j]));
+                next(7, true);
+#pragma unroll
+                for (int j = 0; j < EC; j++) L[j] = both(r0[j], r1[j]);                       // 7, 8
+                next(9, true);
+                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                __syncwarp();
+                if (lane == 0)
+                    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(tmem_empty)) : "memory");
+#pragma unroll
+                for (int j = 0; j < EC; j++) L[j] = (L[j] << 14) + both(r0[j], r1[j]);        // 9, 10
+                if (rok) {
+#pragma unroll
+                    for (int j0 = 0; j0 < EC; j0 += 8) {
+                        double cv[8];
+#pragma unroll
+                        for (int j = 0; j < 8; j++) {
+                            const int col = n0 + cbase + j0 + j;
+                            cv[j] = col < N ? C[row + (int64_t)col * ldc] : 0.0;
+                        }
+#pragma unroll
+                        for (int j = 0; j < 8; j++) {
+                            const int col = n0 + cbase + j0 + j;
+                            if (col < N) {
+                                const int ef = fb[col];
+                                const double v = ::fma(double_of(H[j0 + j]), 0x1p28, double_of(L[j0 + j]));
+                                C[row + (int64_t)col * ldc] =
+                                    (er >= kBadExp || ef >= kBadExp) ? NAN : sub_scaled(cv[j], v, er + ef - 7 * (S + 1));
+                            }
+                        }
+                    }
+                }
+                continue;
+            } else {
             // fold sum_t acc_t 2^(-7 t) into pairs (h, l), exactly term by
             // term, one accumulator (EC columns) at a time.  Two register
             // buffers: the next accumulator's TMEM load is issued before the
@@ -411,7 +543,7 @@ oz_update_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
             uint32_t r0[EC], r1[EC];
             tmem_ld32(base, r0);
             tmem_wait32(r0);
-            tmem_ld32(base + (uint32_t)BN, r1);
+            tmem_ld32(base + (uint32_t)BN<S>, r1);
 #pragma unroll
             for (int j = 0; j < EC; j++) {
                 h[j] = __uint_as_float(r0[j]) * pow2f(-2 * BETA);
@@ -422,7 +554,7 @@ oz_update_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
                 uint32_t(&cur)[EC] = (t & 1) ? r1 : r0;
                 uint32_t(&nxt)[EC] = (t & 1) ? r0 : r1;
                 tmem_wait32(cur);
-                if (t + 1 < S) tmem_ld32(base + (uint32_t)((t + 1) * BN), nxt);
+                if (t + 1 < S) tmem_ld32(base + (uint32_t)((t + 1) * BN<S>), nxt);
                 if (t == S - 1) {
                     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
                     __syncwarp();
@@ -458,6 +590,7 @@ oz_update_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
                         }
                     }
                 }
+            }
             }
         }
     }
@@ -504,6 +637,33 @@ template <int S> __device__ __forceinline__ void digits(df64 v, int e, int (&d)[
     d[0] = high;
 }
 
+// Balanced base-128 digits of round(v 2^(63 - e)), |v| < 2^(e-1), v double: the
+// significand shifted to an integer of at most 62 bits (rounded only where
+// bits fall below 2^(e - 63)), its digits from three 32-bit parts (28 bits,
+// 28 bits and the rest) with a carry from each to the next.
+template <int S> __device__ __forceinline__ void digits(double v, int e, int (&d)[S])
+{
+    static_assert(S == kDigits64 && BETA == 7, "two parts of four digits and a leading one");
+    const long long bits = __double_as_longlong(v);
+    const int ex = (int)(bits >> 52) & 0x7FF;
+    const long long m = (bits & 0xFFFFFFFFFFFFFll) | (ex ? 1ll << 52 : 0ll);
+    const int sh = (ex ? ex : 1) - 1075 + S * BETA - e;  // at most 9
+    long long y = sh >= 0 ? m << sh : (sh > -60 ? (m + (1ll << (-sh - 1))) >> -sh : 0ll);
+    if (bits < 0) y = -y;
+    int part[3] = {(int)(y & 0xFFFFFFF), (int)((y >> 28) & 0xFFFFFFF), (int)(y >> 56)};
+#pragma unroll
+    for (int h = 0; h < 2; h++) {
+#pragma unroll
+        for (int p = S - 1 - 4 * h; p >= S - 4 - 4 * h; p--) {
+            const int r = ((part[h] & 127) ^ 64) - 64;  // -64 .. 63
+            d[p] = r;
+            part[h] = (part[h] - r) >> BETA;
+        }
+        part[h + 1] += part[h];
+    }
+    d[0] = part[2];
+}
+
 // A digit (an integer of at most 8 significant bits) as a bf16: it is exact in
 // float (2^23 + 2^22 + r - (2^23 + 2^22) in float arithmetic), and its float's
 // upper half is then the exact bf16.
@@ -525,13 +685,30 @@ __device__ __forceinline__ int exp_of(float x)
     return e;
 }
 
+__device__ __forceinline__ int exp_of(df64 x) { return exp_of(x.hi); }
+
+// The same for a double (subnormals included); kBadExp for Inf and NaN: a row
+// of A or a column of B that holds one makes its row or column of C NaN, as
+// the products would (an exact zero's product with it is NaN too).
+__device__ __forceinline__ int exp_of(double x)
+{
+    const long long m = __double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFll;
+    const int ex = (int)(m >> 52);
+    if (ex == 0x7FF) return kBadExp;
+    if (m == 0) return kNoExp;
+    return ex ? ex - 1022 : 64 - __clzll(m) - 1074;
+}
+
+__device__ __forceinline__ int finite_exp(int e) { return e == kBadExp ? kNoExp : e; }
+
 // k-balancing exponents, stored as atomicMax targets (initialized to kNoExp):
 // ka[k] = max over rows of E(A_ik), kb[k] = max over columns of E(B_kj).
 // One launch for both: blocks [0, na) take A (block b: column k = b / ca,
 // rows of chunk b % ca, 4096 rows each), the rest take B (64 columns each;
 // threads over k, K <= 512: two per thread at most).
-__global__ void __launch_bounds__(256) kexp_kernel(int M, int K, int N, int ca, int na, const df64 *__restrict__ A,
-                                                   int64_t lda, const df64 *__restrict__ B, int64_t ldb, int *ka,
+template <typename TE>
+__global__ void __launch_bounds__(256) kexp_kernel(int M, int K, int N, int ca, int na, const TE *__restrict__ A,
+                                                   int64_t lda, const TE *__restrict__ B, int64_t ldb, int *ka,
                                                    int *kb)
 {
     const int b = blockIdx.x;
@@ -539,7 +716,7 @@ __global__ void __launch_bounds__(256) kexp_kernel(int M, int K, int N, int ca, 
         const int k = b / ca, chunk = b % ca;
         int e = kNoExp;
         const int r1 = min(M, (chunk + 1) * 4096);
-        for (int r = chunk * 4096 + threadIdx.x; r < r1; r += 256) e = max(e, exp_of(A[r + (int64_t)k * lda].hi));
+        for (int r = chunk * 4096 + threadIdx.x; r < r1; r += 256) e = max(e, finite_exp(exp_of(A[r + (int64_t)k * lda])));
         for (int o = 16; o > 0; o >>= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
         if (threadIdx.x % 32 == 0 && e > kNoExp) atomicMax(ka + k, e);
         return;
@@ -547,7 +724,7 @@ __global__ void __launch_bounds__(256) kexp_kernel(int M, int K, int N, int ca, 
     const int c0 = (b - na) * 64, c1 = min(N, c0 + 64);
     for (int k = threadIdx.x; k < K; k += 256) {
         int e = kNoExp;
-        for (int c = c0; c < c1; c++) e = max(e, exp_of(B[k + (int64_t)c * ldb].hi));
+        for (int c = c0; c < c1; c++) e = max(e, finite_exp(exp_of(B[k + (int64_t)c * ldb])));
         if (e > kNoExp) atomicMax(kb + k, e);
     }
 }
@@ -567,20 +744,20 @@ __device__ __forceinline__ int kshift(const int *ka, const int *kb, int k)
 // a 32 x 32 shared tile: loaded with consecutive threads down a column of A,
 // written with consecutive threads along k of one output row.
 template <int S>
-__device__ __forceinline__ void slice_rows_block(int blk, int M, int K, int Kp, int Mp, const df64 *__restrict__ A,
+__device__ __forceinline__ void slice_rows_block(int blk, int M, int K, int Kp, int Mp, const elem_t<S> *__restrict__ A,
                                                  int64_t lda, const int *__restrict__ ka, const int *__restrict__ kb,
                                                  __nv_bfloat16 *out, int *ea)
 {
     __shared__ int smax[32][9];
     __shared__ int sexp[32];
-    __shared__ df64 tile[32][33];
+    __shared__ elem_t<S> tile[32][33];
     const int r = threadIdx.x % 32, kl = threadIdx.x / 32;  // 32 rows x 8 lanes of K
     const int m = blk * 32 + r;
     int emax = kNoExp;  // max over k of E(A_mk 2^t_k)
     if (m < M)
         for (int k = kl; k < K; k += 8) {
-            const int e = exp_of(A[m + (int64_t)k * lda].hi);
-            if (e != kNoExp) emax = max(emax, e + kshift(ka, kb, k));
+            const int e = exp_of(A[m + (int64_t)k * lda]);
+            if (e != kNoExp) emax = max(emax, e == kBadExp ? e : e + kshift(ka, kb, k));
         }
     smax[r][kl] = emax;
     __syncthreads();
@@ -588,7 +765,7 @@ __device__ __forceinline__ void slice_rows_block(int blk, int M, int K, int Kp, 
         int mx = kNoExp;
         for (int j = 0; j < 8; j++) mx = max(mx, smax[threadIdx.x][j]);
         // the pair's low part can push |hi + lo| just past a power of two: one more bit of headroom
-        int e = mx == kNoExp ? 0 : mx + 1;
+        int e = mx == kNoExp ? 0 : (mx == kBadExp ? mx : mx + 1);
         sexp[threadIdx.x] = e;
         int mm = blk * 32 + threadIdx.x;
         if (mm < M) ea[mm] = e;
@@ -599,7 +776,7 @@ __device__ __forceinline__ void slice_rows_block(int blk, int M, int K, int Kp, 
 #pragma unroll
         for (int j = 0; j < 4; j++) {
             const int k = k0 + kl + 8 * j;
-            tile[r][kl + 8 * j] = (m < M && k < K) ? A[m + (int64_t)k * lda] : df64(0.f, 0.f);
+            tile[r][kl + 8 * j] = (m < M && k < K) ? A[m + (int64_t)k * lda] : elem_t<S>(0);
         }
         __syncthreads();
         const int k = k0 + kk;
@@ -609,8 +786,8 @@ __device__ __forceinline__ void slice_rows_block(int blk, int M, int K, int Kp, 
             const int mm = blk * 32 + rr;
             if (mm >= Mp) continue;
             int d[S];
-            if (mm < M && k < K) {
-                digits(tile[rr][kk], sexp[rr] - kshift(ka, kb, k), d);
+            if (mm < M && k < K && sexp[rr] != kBadExp) {
+                digits<S>(tile[rr][kk], sexp[rr] - kshift(ka, kb, k), d);
             } else {
 #pragma unroll
                 for (int p = 0; p < S; p++) d[p] = 0;
@@ -624,7 +801,7 @@ __device__ __forceinline__ void slice_rows_block(int blk, int M, int K, int Kp, 
 // B (K x N df64, column-major ldb) -> digit slices of B^T (rows n, K-major), column exponents.
 // One warp per column.
 template <int S>
-__device__ __forceinline__ void slice_cols_warp(int n, int K, int N, int Kp, int Np, const df64 *__restrict__ B,
+__device__ __forceinline__ void slice_cols_warp(int n, int K, int N, int Kp, int Np, const elem_t<S> *__restrict__ B,
                                                 int64_t ldb, const int *__restrict__ ka, const int *__restrict__ kb,
                                                 __nv_bfloat16 *out, int *fb)
 {
@@ -633,16 +810,16 @@ __device__ __forceinline__ void slice_cols_warp(int n, int K, int N, int Kp, int
     int emax = kNoExp;  // max over k of E(B_kn 2^-t_k)
     if (n < N)
         for (int k = lane; k < K; k += 32) {
-            const int e = exp_of(B[k + (int64_t)n * ldb].hi);
-            if (e != kNoExp) emax = max(emax, e - kshift(ka, kb, k));
+            const int e = exp_of(B[k + (int64_t)n * ldb]);
+            if (e != kNoExp) emax = max(emax, e == kBadExp ? e : e - kshift(ka, kb, k));
         }
     for (int o = 16; o > 0; o >>= 1) emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, o));
-    const int e = emax == kNoExp ? 0 : emax + 1;
+    const int e = emax == kNoExp ? 0 : (emax == kBadExp ? emax : emax + 1);
     if (lane == 0 && n < N) fb[n] = e;
     for (int k = lane; k < Kp; k += 32) {
         int d[S];
-        if (n < N && k < K) {
-            digits(B[k + (int64_t)n * ldb], e + kshift(ka, kb, k), d);
+        if (n < N && k < K && e != kBadExp) {
+            digits<S>(B[k + (int64_t)n * ldb], e + kshift(ka, kb, k), d);
         } else {
 #pragma unroll
             for (int p = 0; p < S; p++) d[p] = 0;
@@ -656,8 +833,8 @@ __device__ __forceinline__ void slice_cols_warp(int n, int K, int N, int Kp, int
 // rest slice 8 columns of B each (one warp per column).
 template <int S>
 __global__ void __launch_bounds__(256, 4) slice_kernel(int M, int N, int K, int Kp, int Mp, int Np, int nra,
-                                                    const df64 *__restrict__ A, int64_t lda,
-                                                    const df64 *__restrict__ B, int64_t ldb,
+                                                    const elem_t<S> *__restrict__ A, int64_t lda,
+                                                    const elem_t<S> *__restrict__ B, int64_t ldb,
                                                     const int *__restrict__ ka, const int *__restrict__ kb,
                                                     __nv_bfloat16 *sa, int *ea, __nv_bfloat16 *sb, int *fb)
 {
@@ -712,7 +889,7 @@ size_t oz_update_workspace(int64_t M, int64_t N, int64_t K, int digits)
 {
     using namespace oz;
     const int64_t S = digits;
-    const int64_t Mp = rup(M, BM), Np = rup(N, BN), Kp = rup(K, KSLAB);
+    const int64_t Mp = rup(M, BM), Np = rup(N, digits == kDigits64 ? BN<9> : BN<8>), Kp = rup(K, KSLAB);
     return (size_t)rup(S * Mp * Kp * 2, 1024) + (size_t)rup(S * Np * Kp * 2, 1024) + (size_t)rup(Mp * 4, 256) +
            (size_t)rup(Np * 4, 256) + 2 * (size_t)rup(Kp * 4, 256) + 256;
 }
@@ -736,14 +913,14 @@ struct Slices {
     int64_t M, N, K, Mp, Np, Kp;
 };
 
-static Slices carve(int64_t M, int64_t N, int64_t K, int S, void *work)
+template <int S> static Slices carve(int64_t M, int64_t N, int64_t K, void *work)
 {
     Slices sl;
     sl.M = M;
     sl.N = N;
     sl.K = K;
     sl.Mp = rup(M, BM);
-    sl.Np = rup(N, BN);
+    sl.Np = rup(N, BN<S>);
     sl.Kp = rup(K, KSLAB);
     char *w = (char *)work;
     sl.sa = (__nv_bfloat16 *)w;
@@ -762,7 +939,8 @@ static Slices carve(int64_t M, int64_t N, int64_t K, int S, void *work)
 
 // The balancing exponents and digit slices of A (M x K) and B (K x N).
 template <int S>
-static rbt_status slice(const Slices &sl, const df64 *A, int64_t lda, const df64 *B, int64_t ldb, cudaStream_t stream)
+static rbt_status slice(const Slices &sl, const elem_t<S> *A, int64_t lda, const elem_t<S> *B, int64_t ldb,
+                        cudaStream_t stream)
 {
     const int64_t M = sl.M, N = sl.N, K = sl.K;
     if (M <= 0 || N <= 0 || K <= 0) return RBT_OK;
@@ -770,7 +948,7 @@ static rbt_status slice(const Slices &sl, const df64 *A, int64_t lda, const df64
     // both exponent arrays start at kNoExp (every byte 0x80)
     RBT_CUDA_TRY(cudaMemsetAsync(sl.ka, 0x80, (size_t)rup(sl.Kp * 4, 256) * 2, stream));
     const int ca = (int)cdiv(M, 4096), na = ca * (int)K;
-    kexp_kernel<<<(unsigned)(na + cdiv(N, 64)), 256, 0, stream>>>((int)M, (int)K, (int)N, ca, na, A, lda, B, ldb,
+    kexp_kernel<elem_t<S>><<<(unsigned)(na + cdiv(N, 64)), 256, 0, stream>>>((int)M, (int)K, (int)N, ca, na, A, lda, B, ldb,
                                                                     sl.ka, sl.kb);
     RBT_LAUNCH_CHECK();
     const int nra = (int)cdiv(sl.Mp, 32);
@@ -785,16 +963,16 @@ static rbt_status slice(const Slices &sl, const df64 *A, int64_t lda, const df64
 // B from the slices (a0 a multiple of BM, b0 of BN, both blocks inside the
 // sliced product), on at most max_ctas CTAs.
 template <int S>
-static rbt_status multiply(const Slices &sl, int64_t a0, int64_t b0, int64_t Ms, int64_t Ns, df64 *C, int64_t ldc,
+static rbt_status multiply(const Slices &sl, int64_t a0, int64_t b0, int64_t Ms, int64_t Ns, elem_t<S> *C, int64_t ldc,
                            const int64_t *info, void *status, unsigned max_ctas, cudaStream_t stream)
 {
     if (Ms <= 0 || Ns <= 0) return RBT_OK;
-    if (a0 % BM || b0 % BN || a0 < 0 || b0 < 0 || a0 + Ms > sl.M || b0 + Ns > sl.N) return RBT_ERR_ARG;
+    if (a0 % BM || b0 % BN<S> || a0 < 0 || b0 < 0 || a0 + Ms > sl.M || b0 + Ns > sl.N) return RBT_ERR_ARG;
     ProfScope ps(kProfUpdate, stream);
     CUtensorMap ma, mb;
-    if (!make_map(&ma, sl.sa, (int)(S * sl.Mp), (int)sl.Kp, BM) || !make_map(&mb, sl.sb, (int)(S * sl.Np), (int)sl.Kp, BN))
+    if (!make_map(&ma, sl.sa, (int)(S * sl.Mp), (int)sl.Kp, BM) || !make_map(&mb, sl.sb, (int)(S * sl.Np), (int)sl.Kp, BN<S>))
         return RBT_ERR_CUDA;
-    const int64_t ntiles = cdiv(Ms, BM) * cdiv(Ns, BN);
+    const int64_t ntiles = cdiv(Ms, BM) * cdiv(Ns, BN<S>);
     const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(ntiles, max_ctas));
     oz_update_kernel<false, S><<<grid, kOzThreads, kSmemBytes<S>, stream>>>(
         ma, mb, (int)Ms, (int)Ns, (int)sl.Kp, (int)sl.Mp, (int)sl.Np, (int)a0, (int)b0, sl.ea + a0, sl.fb + b0, C,
@@ -804,14 +982,14 @@ static rbt_status multiply(const Slices &sl, int64_t a0, int64_t b0, int64_t Ms,
 }
 
 template <int S>
-static rbt_status update(int64_t M, int64_t N, int64_t K, const df64 *A, int64_t lda, const df64 *B, int64_t ldb,
-                         df64 *C, int64_t ldc, const int64_t *info, void *work, void *status, unsigned max_ctas,
+static rbt_status update(int64_t M, int64_t N, int64_t K, const elem_t<S> *A, int64_t lda, const elem_t<S> *B,
+                         int64_t ldb, elem_t<S> *C, int64_t ldc, const int64_t *info, void *work, void *status, unsigned max_ctas,
                          cudaStream_t stream)
 {
     if (M <= 0 || N <= 0 || K <= 0) return RBT_OK;
     rbt_status s = configure<S>();
     if (s != RBT_OK) return s;
-    const Slices sl = carve(M, N, K, S, work);
+    const Slices sl = carve<S>(M, N, K, work);
     s = slice<S>(sl, A, lda, B, ldb, stream);
     if (s != RBT_OK) return s;
     return multiply<S>(sl, 0, 0, M, N, C, ldc, info, status, max_ctas, stream);
@@ -828,7 +1006,7 @@ rbt_status oz_update(int64_t M, int64_t N, int64_t K, const df64 *A, int64_t lda
     using namespace oz;
     if (M <= 0 || N <= 0 || K <= 0) return RBT_OK;
     if (digits != 7 && digits != 8) return RBT_ERR_ARG;
-    if (K > KMAX || M > INT32_MAX / digits || N > INT32_MAX / digits) return RBT_ERR_UNSUPPORTED;
+    if (K > KMAX<8> || M > INT32_MAX / digits || N > INT32_MAX / digits) return RBT_ERR_UNSUPPORTED;
     if (work_bytes < oz_update_workspace(M, N, K, digits)) return RBT_ERR_WORKSPACE;
     const unsigned ctas = max_ctas ? max_ctas : (unsigned)device_sm_count();
     return digits == 7 ? update<7>(M, N, K, A, lda, B, ldb, C, ldc, info, work, status, ctas, stream)
@@ -868,7 +1046,7 @@ size_t oz_products_workspace(int64_t M, int64_t N, int64_t K)
 {
     using namespace oz;
     if (M <= 0 || N <= 0 || K <= 0) return 0;
-    const int64_t Mp = rup(M, BM), Np = rup(N, BN), Kp = rup(K, KSLAB);
+    const int64_t Mp = rup(M, BM), Np = rup(N, BN<kRawDigits>), Kp = rup(K, KSLAB);
     return (size_t)rup(kRawDigits * Mp * Kp * 2, 1024) + (size_t)rup(kRawDigits * Np * Kp * 2, 1024) + 256;
 }
 
@@ -881,11 +1059,11 @@ rbt_status oz_products(int64_t M, int64_t N, int64_t K, const int8_t *da, const 
     if (M < 0 || N < 0 || K < 0) return RBT_ERR_ARG;
     if (M == 0 || N == 0 || K == 0) return RBT_OK;
     if (!da || !db || !acc) return RBT_ERR_ARG;
-    if (K > KMAX || M > INT32_MAX / kRawDigits || N > INT32_MAX / kRawDigits) return RBT_ERR_UNSUPPORTED;
+    if (K > KMAX<kRawDigits> || M > INT32_MAX / kRawDigits || N > INT32_MAX / kRawDigits) return RBT_ERR_UNSUPPORTED;
     if (!work || work_bytes < oz_products_workspace(M, N, K)) return RBT_ERR_WORKSPACE;
     rbt_status s = configure<kRawDigits>();
     if (s != RBT_OK) return s;
-    const int64_t Mp = rup(M, BM), Np = rup(N, BN), Kp = rup(K, KSLAB);
+    const int64_t Mp = rup(M, BM), Np = rup(N, BN<kRawDigits>), Kp = rup(K, KSLAB);
     char *w = (char *)work;
     __nv_bfloat16 *sa = (__nv_bfloat16 *)w;
     w += rup(kRawDigits * Mp * Kp * 2, 1024);
@@ -901,9 +1079,9 @@ rbt_status oz_products(int64_t M, int64_t N, int64_t K, const int8_t *da, const 
     digits_to_slices_kernel<<<(unsigned)cdiv(tb, 256), 256, 0, stream>>>((int)N, (int)Np, (int)K, (int)Kp, db, sb);
     RBT_LAUNCH_CHECK();
     CUtensorMap ma, mb;
-    if (!make_map(&ma, sa, (int)(kRawDigits * Mp), (int)Kp, BM) || !make_map(&mb, sb, (int)(kRawDigits * Np), (int)Kp, BN))
+    if (!make_map(&ma, sa, (int)(kRawDigits * Mp), (int)Kp, BM) || !make_map(&mb, sb, (int)(kRawDigits * Np), (int)Kp, BN<kRawDigits>))
         return RBT_ERR_CUDA;
-    const int64_t ntiles = (Mp / BM) * (Np / BN);
+    const int64_t ntiles = (Mp / BM) * (Np / BN<kRawDigits>);
     const unsigned grid = (unsigned)std::min<int64_t>(ntiles, device_sm_count());
     oz_update_kernel<true, kRawDigits><<<grid, kOzThreads, kSmemBytes<kRawDigits>, stream>>>(ma, mb, (int)M, (int)N, (int)Kp, (int)Mp,
                                                                      (int)Np, 0, 0, nullptr, nullptr, nullptr, 0, info,
@@ -931,13 +1109,14 @@ rbt_status rbt_debug_oz_products(int64_t M, int64_t N, int64_t K, const int8_t *
 
 namespace rbt {
 
-constexpr int kOzOuterNB = 512;  // K of the trailing update (digit-product exactness bound)
+// K of the trailing update: the digit-product exactness bound
 constexpr int kOzInnerNB = 64;   // panel step (double-float diagonal factor and TRSMs)
 
 size_t oz_factor_workspace(int64_t n)
 {
     if (n <= 0) return 0;
-    return oz_update_workspace(n, n, kOzOuterNB, oz::kMaxDigits) + 256;  // any digit count
+    // any digit count
+    return std::max(oz_update_workspace(n, n, oz::KMAX<8>, 8), oz_update_workspace(n, n, oz::KMAX<9>, 9)) + 256;
 }
 
 namespace {
@@ -948,9 +1127,10 @@ namespace {
 // to its right), then one rank-512 sliced tensor-core update of the trailing
 // matrix per panel.
 template <int S>
-rbt_status factor_oz(int64_t n, df64 *A, int64_t lda, int64_t *info, void *work, cudaStream_t stream)
+rbt_status factor_oz(int64_t n, oz::elem_t<S> *A, int64_t lda, int64_t *info, void *work, cudaStream_t stream)
 {
-    const size_t ws = oz_update_workspace(n, n, kOzOuterNB, oz::kMaxDigits);
+    constexpr int kOzOuterNB = oz::KMAX<S>;
+    const size_t ws = oz_factor_workspace(n) - 256;
     void *status = (char *)work + ws;
     RBT_CUDA_TRY(cudaMemsetAsync(status, 0, 256, stream));
     const unsigned sms = (unsigned)device_sm_count();
@@ -959,7 +1139,7 @@ rbt_status factor_oz(int64_t n, df64 *A, int64_t lda, int64_t *info, void *work,
         const int64_t kb = n - k < kOzOuterNB ? n - k : kOzOuterNB;
         for (int64_t j = k; j < k + kb; j += kOzInnerNB) {
             const int jb = (int)(k + kb - j < kOzInnerNB ? k + kb - j : kOzInnerNB);
-            s = genp_panel_steps<df64>(n, A, lda, info, jb, j, j + jb, false, stream);
+            s = genp_panel_steps<oz::elem_t<S>>(n, A, lda, info, jb, j, j + jb, false, stream);
             if (s != RBT_OK) return s;
             const int64_t r0 = j + jb;
             s = oz::update<S>(n - r0, k + kb - r0, jb, A + r0 + j * lda, lda, A + j + r0 * lda, lda,
@@ -978,6 +1158,14 @@ rbt_status factor_oz(int64_t n, df64 *A, int64_t lda, int64_t *info, void *work,
 }
 
 }  // namespace
+
+rbt_status genp_factor_oz64(int64_t n, double *A, int64_t lda, int64_t *info, void *work, size_t work_bytes,
+                            cudaStream_t stream)
+{
+    if (work_bytes < oz_factor_workspace(n) || !work) return RBT_ERR_WORKSPACE;
+    if (n > INT32_MAX / oz::kDigits64) return RBT_ERR_UNSUPPORTED;
+    return factor_oz<oz::kDigits64>(n, A, lda, info, work, stream);
+}
 
 // digits = 7 or 8 per entry of the sliced operands
 rbt_status genp_factor_oz(int64_t n, df64 *A, int64_t lda, int64_t *info, void *work, size_t work_bytes, int digits,

@@ -24,6 +24,8 @@ rbt_status oz_update(int64_t M, int64_t N, int64_t K, const df64 *A, int64_t lda
                      cudaStream_t stream, unsigned max_ctas = 0);
 rbt_status oz_status_to_info(void *status, int64_t *info, cudaStream_t stream);
 size_t oz_factor_workspace(int64_t n);
+rbt_status genp_factor_oz64(int64_t n, double *A, int64_t lda, int64_t *info, void *work, size_t work_bytes,
+                            cudaStream_t stream);
 rbt_status genp_factor_oz(int64_t n, df64 *A, int64_t lda, int64_t *info, void *work, size_t work_bytes, int digits,
                           cudaStream_t stream);
 

@@ -73,7 +73,12 @@ rbt_status genp_solve_wp_run(int64_t n, int64_t nrhs, int32_t prec, const void *
                              double *B, int64_t ldb, void *work, bool have_inv, cudaStream_t stream);
 
 size_t genp_factor_workspace_impl(int64_t n, int prec, int nb);
+
+// Whether every row and column of a double matrix has mostly entries of like
+// size (spread.cu); scratch: spread_workspace(n) bytes.  Synchronizes.
+size_t spread_workspace(int64_t n);
+rbt_status evenly_spread(int64_t n, const double *A, int64_t lda, void *scratch, bool *even, cudaStream_t stream);
 rbt_status genp_factor_impl(int64_t n, int prec, void *A, int64_t lda, int64_t *info, void *work,
-                            size_t work_bytes, int nb, cudaStream_t stream);
+                            size_t work_bytes, int nb, cudaStream_t stream, bool sliced64 = false);
 
 }  // namespace rbt
