@@ -62,11 +62,13 @@ __device__ __forceinline__ double to_double(float v) { return (double)v; }
 __device__ __forceinline__ double to_double(df64 v) { return df_to_double(v); }
 
 // A running sum of products.  Double-float: the leading part stays exact by
-// TwoSum and every error term gathers in a float, 12 FP32 operations a
-// multiply-add and one dependent addition a step.  The gathered float is
-// folded in after every block's few terms: left to grow over a whole row its
-// own rounding grows with the number of terms (first backward error of an
-// n = 40003 solve 2.8e-8, folded 9.7e-10).
+// TwoSum; its errors gather in one float and the products' own errors and
+// cross terms, smaller by the ratio of a product to the sum, in another: 12
+// FP32 operations a multiply-add, one dependent addition a step, and one
+// rounding at the sum's scale.  Both floats are folded in after every block's
+// few terms (left to grow over a whole row their own rounding grows with the
+// number of terms: first backward error of an n = 40003 solve 2.8e-8 instead
+// of 9.6e-10).
 template <typename T> struct Acc {
     T s = T(0);
     __device__ __forceinline__ void mac(T a, T b) { s = fma(a, b, s); }
@@ -74,7 +76,7 @@ template <typename T> struct Acc {
     __device__ __forceinline__ T value() const { return s; }
 };
 template <> struct Acc<df64> {
-    float h = 0.f, l = 0.f;
+    float h = 0.f, l = 0.f, c = 0.f;
     __device__ __forceinline__ void mac(df64 a, df64 b)
     {
         const float p = __fmul_rn(a.hi, b.hi);
@@ -82,10 +84,15 @@ template <> struct Acc<df64> {
         float s, e;
         two_sum(h, p, s, e);
         h = s;
-        l = __fmaf_rn(a.lo, b.hi, __fmaf_rn(a.hi, b.lo, __fadd_rn(l, __fadd_rn(e, pe))));
+        l = __fadd_rn(l, e);
+        c = __fmaf_rn(a.lo, b.hi, __fmaf_rn(a.hi, b.lo, __fadd_rn(c, pe)));
     }
-    __device__ __forceinline__ void fold() { fast_two_sum(h, l, h, l); }
-    __device__ __forceinline__ df64 value() const { return df_norm(h, l); }
+    __device__ __forceinline__ void fold()
+    {
+        fast_two_sum(h, __fadd_rn(l, c), h, l);
+        c = 0.f;
+    }
+    __device__ __forceinline__ df64 value() const { return df_norm(h, __fadd_rn(l, c)); }
 };
 
 // ---- published values
