@@ -509,7 +509,7 @@ def run_ours(args):
     peaks, peak_src = measured_peaks()
     nb = args.nb or (64 if prec in ("f64", "df64") else 128)
     upd_ms, upd_n = prof["update"]
-    # df64tc: 512-column panels factored in 64-column steps, every update of
+    # df64tc: 512-column panels (df64tc7: 448) factored in 64-column steps, every update of
     # both levels on the sliced kernel, so the update class does all the
     # flops of 64-column blocking
     upd_flops = update_flops(n, nb if prec not in DIGIT_PRODUCTS else 64) * args.steps
@@ -558,7 +558,7 @@ def run_ours(args):
              "df64tc": "oz_update_kernel<8>", "df64tc7": "oz_update_kernel<7>"}.get(prec, "gemm_sub_kernel")
     es = {"df64": 8, "f64": 8, "df64tc": 8, "df64tc7": 8}.get(prec, 4)
     ratio = traffic_ratio(kname)
-    alg_bytes = oz_update_bytes(n) if prec in DIGIT_PRODUCTS else update_bytes(n, nb, es)
+    alg_bytes = oz_update_bytes(n, outer=448 if prec == "df64tc7" else 512) if prec in DIGIT_PRODUCTS else update_bytes(n, nb, es)
     alg_per_launch = alg_bytes * args.steps / max(upd_n, 1)
     roof.update({"kernel": "genp trailing update (%s)" % kname, "achieved": achieved,
                  "frac": (achieved / roof["peak"]) if achieved else None,
@@ -598,7 +598,7 @@ def run_ours(args):
         "warmup": max(3, args.warmup), "ms_per_step": ms, "higher_is_better": True, "scaling": "weak",
         "vs_baseline": None, "dtype": "%s+f64" % prec, "data": "synthetic",
         "config": {"workload": "rbt_genp_solve_precision", "n": n, "d": d, "nrhs": 1,
-                   "matrix": "D_r G D_c, G~N(0,1), D=10^U(-1.5,1.5)", "prec": prec, "nb": nb if prec not in DIGIT_PRODUCTS else "512/64",
+                   "matrix": "D_r G D_c, G~N(0,1), D=10^U(-1.5,1.5)", "prec": prec, "nb": nb if prec not in DIGIT_PRODUCTS else "448/64" if prec == "df64tc7" else "512/64",
                    "refine": "FP64 IR to berr<=1e-13, %s on stall" % ("eight-digit then FP64 refactor"
                                                                         if prec == "df64tc7" else "FP64 refactor"),
                    "l2": "inputs 12.8 GB >> L2, no flush",

@@ -58,16 +58,15 @@
 
 #include <algorithm>
 #include <mutex>
-#include <type_traits>
 
 #include "df64.cuh"
 #include "gemm_tc.cuh"
 #include "genp_internal.cuh"
+#include "oz_slice.cuh"
 
 namespace rbt {
 namespace oz {
 
-constexpr int BETA = 7;     // bits per digit
 constexpr int BM = 128;
 // TMEM holds one 128 x BN FP32 accumulator per digit weight t = 2 .. S + 1 in
 // 512 columns: 64 columns each for S = 7 and 8, 48 for S = 9.
@@ -89,24 +88,23 @@ constexpr int TMEM_COLS = 512;
 // a digit product is at most 64 * 64 = 2^12 and a weight holds at most S of
 // them per k: S * K * 2^12 <= 2^24 keeps every accumulation exact
 template <int S> constexpr int KMAX = S <= 8 ? 512 : 448;
+// the factorizations' panels: with seven digits the leading one is wide
+// (oz_slice.cuh), (S + 2) K 2^12 <= 2^24
+template <int S> constexpr bool kWide = S == 7;
+template <int S> constexpr int kOuterNB = kWide<S> ? 448 : KMAX<S>;
 constexpr int kMaxDigits = 8;    // of double-float operands
-constexpr int kDigits64 = 9;     // of double operands: 63 bits
-static_assert(kMaxDigits * KMAX<8> * 4096 <= (1 << 24) && kDigits64 * KMAX<9> * 4096 <= (1 << 24),
+static_assert(kMaxDigits * KMAX<8> * 4096 <= (1 << 24) && kDigits64 * KMAX<9> * 4096 <= (1 << 24) &&
+                  (7 + 2) * kOuterNB<7> * 4096 <= (1 << 24),
               "digit accumulation must stay exact");
 static_assert(kMaxDigits * BN<8> <= TMEM_COLS && kDigits64 * BN<9> <= TMEM_COLS,
               "one accumulator per digit weight in TMEM");
 static_assert(kStages<9> >= 2 && kStages<8> >= 2 && kStages<7> >= 2, "at least double buffering");
-// digits of an operand type's updates and back
-template <int S> using elem_t = std::conditional_t<S == kDigits64, double, df64>;
 constexpr int kGroupM = 16;  // row tiles per group of the tile order (L2 reuse of the digit slices)
 
 struct Status {
     int err;
 };
 
-// exponent of a row or column with an entry that is not finite (double
-// operands), above every exponent that occurs
-constexpr int kBadExp = 1 << 28;
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -265,31 +263,44 @@ __device__ __forceinline__ bool mbar_wait_ab(uint64_t *bar, uint32_t parity, Sta
     return true;
 }
 
-// Output tile i of this CTA (tiles dealt round-robin over the grid, in the
-// grouped order below).  Groups of kGroupM row tiles, columns outer and rows
-// inner within a group: the tiles in flight at one time share a band of
-// kGroupM x 128 rows of A's digit slices and a few column tiles of B's, both
-// L2-resident, instead of every wave streaming A's slices from DRAM.
-__device__ __forceinline__ void tile_origin(int64_t i, int tiles_m, int tiles_n, int bn, int &m0, int &n0)
+// One product of a launch: C (M x N, ldc) -= A B from the digit slices (padded
+// row counts Mp, Np of one slice) and the row / column exponents.
+template <int S> struct Problem {
+    int M, N, Mp, Np;
+    const int *ea, *fb;
+    elem_t<S> *C;
+    int64_t ldc;
+    int tiles_m, tiles_n;
+    int64_t ntiles;
+};
+
+// Output tile i of this CTA: tiles dealt round-robin over the grid, the first
+// problem's before the second's, in a grouped order.  Groups of kGroupM row
+// tiles, columns outer and rows inner within a group: the tiles in flight at
+// one time share a band of kGroupM x 128 rows of A's digit slices and a few
+// column tiles of B's, both L2-resident, instead of every wave streaming A's
+// slices from DRAM.  Returns the problem.
+template <int S>
+__device__ __forceinline__ int tile_origin(int64_t i, const Problem<S> &p0, const Problem<S> &p1, int &m0, int &n0)
 {
-    const int64_t t = blockIdx.x + i * gridDim.x;
+    int64_t t = blockIdx.x + i * gridDim.x;
+    const int which = t >= p0.ntiles;
+    if (which) t -= p0.ntiles;
+    const int tiles_m = which ? p1.tiles_m : p0.tiles_m, tiles_n = which ? p1.tiles_n : p0.tiles_n;
     const int64_t per_group = (int64_t)kGroupM * tiles_n;
     const int grp = (int)(t / per_group), in_grp = (int)(t % per_group);
     const int first_m = grp * kGroupM;
     const int gm = tiles_m - first_m < kGroupM ? tiles_m - first_m : kGroupM;
     m0 = (first_m + in_grp % gm) * BM;
-    n0 = (in_grp / gm) * bn;
+    n0 = (in_grp / gm) * BN<S>;
+    return which;
 }
 
-// C (df64, M x N, ldc) -= A B from the digit slices; ea[m] / fb[n] are the
-// row / column exponents.  Every wait gives up after wait_ns (then st->err
-// records the timeout, the other roles stop, and TMEM is freed as usual);
-// with no_copy set (a test stall) the producer issues no copy at all, so the
-// MMA warp's first wait runs out.  A slices: rows p*Mp + a0 + m of the A map,
-// B slices: rows q*Np + b0 + n of the B map (p, q = 0 .. S-1 for digits
-// 1 .. S; Mp, Np the padded row counts of one digit slice, a0 and b0 the
-// first slice row of this block: C may be a sub-block of the sliced product,
-// with ea and fb offset to match).
+// One or two products of the same K (the second may have no tiles), tensor
+// maps of their slices (slice p of A at rows p Mp + m).  Every wait gives up
+// after wait_ns (then st->err records the timeout, the other roles stop, and
+// TMEM is freed as usual); with no_copy set (a test stall) the producer issues
+// no copy at all, so the MMA warp's first wait runs out.
 //
 // Persistent, one CTA per SM, warp-specialized:
 //   warp kProdWarp   (one lane) TMA producer, running ahead over the slabs of
@@ -303,13 +314,13 @@ __device__ __forceinline__ void tile_origin(int64_t i, int tiles_m, int tiles_n,
 // C); the next tile's first slabs are loaded meanwhile, and each tile's
 // block of C is prefetched into L2 while that tile's MMAs run.
 // RAW (testing only): the epilogue writes the S accumulators themselves to
-// raw[(t M + m) N + n] instead of folding them into C (ea, fb, C unused).
+// raw[(t M + m) N + n] of the one problem instead of folding them into C.
 template <bool RAW, int S>
 __global__ void __launch_bounds__(kOzThreads, 1)
-oz_update_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_b, int M,
-                 int N, int K, int Mp, int Np, int a0, int b0, const int *__restrict__ ea, const int *__restrict__ fb,
-                 elem_t<S> *__restrict__ C, int64_t ldc, const int64_t *info, Status *st, long long wait_ns,
-                 int no_copy, float *__restrict__ raw)
+oz_update_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_b,
+                 const __grid_constant__ CUtensorMap tmap_a1, const __grid_constant__ CUtensorMap tmap_b1,
+                 const __grid_constant__ Problem<S> p0, const __grid_constant__ Problem<S> p1, int K,
+                 const int64_t *info, Status *st, long long wait_ns, int no_copy, float *__restrict__ raw)
 {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char *smem = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -324,8 +335,7 @@ oz_update_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
     static_assert(S >= 5 && S <= kDigits64, "digit count");
     if (*((volatile const int64_t *)info) >= 0) return;
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-    const int tiles_m = (M + BM - 1) / BM, tiles_n = (N + BN<S> - 1) / BN<S>;
-    const int64_t ntiles = (int64_t)tiles_m * tiles_n;
+    const int64_t ntiles = p0.ntiles + p1.ntiles;
     if ((int64_t)blockIdx.x >= ntiles) return;
     const int64_t my_tiles = (ntiles - blockIdx.x + gridDim.x - 1) / gridDim.x;
     const int nk = (K + KSLAB - 1) / KSLAB;
@@ -358,7 +368,9 @@ oz_update_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
             int64_t g = 0;
             for (int64_t i = 0; i < my_tiles && !*abort && !no_copy; i++) {
                 int m0, n0;
-                tile_origin(i, tiles_m, tiles_n, BN<S>, m0, n0);
+                const int which = tile_origin<S>(i, p0, p1, m0, n0);
+                const CUtensorMap *ta = which ? &tmap_a1 : &tmap_a, *tb = which ? &tmap_b1 : &tmap_b;
+                const int Mp = which ? p1.Mp : p0.Mp, Np = which ? p1.Np : p0.Np;
                 for (int kt = 0; kt < nk; kt++, g++) {
                     const int s = (int)(g % kStages<S>);
                     const int64_t r = g / kStages<S>;
@@ -369,8 +381,8 @@ oz_update_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
                                  "r"(kStageBytes<S>)
                                  : "memory");
                     for (int p = 0; p < S; p++) {
-                        tma_load_2d(sa + p * A_SLICE_BYTES, &tmap_a, kt * KSLAB, p * Mp + a0 + m0, &full[s]);
-                        tma_load_2d(sb + p * B_SLICE_BYTES<S>, &tmap_b, kt * KSLAB, p * Np + b0 + n0, &full[s]);
+                        tma_load_2d(sa + p * A_SLICE_BYTES, ta, kt * KSLAB, p * Mp + m0, &full[s]);
+                        tma_load_2d(sb + p * B_SLICE_BYTES<S>, tb, kt * KSLAB, p * Np + n0, &full[s]);
                     }
                 }
             }
@@ -433,7 +445,11 @@ oz_update_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
         const uint32_t lane_base = (uint32_t)(q * 32) << 16;
         for (int64_t i = 0; i < my_tiles; i++) {
             int m0, n0;
-            tile_origin(i, tiles_m, tiles_n, BN<S>, m0, n0);
+            const int which = tile_origin<S>(i, p0, p1, m0, n0);
+            const int M = which ? p1.M : p0.M, N = which ? p1.N : p0.N;
+            const int64_t ldc = which ? p1.ldc : p0.ldc;
+            elem_t<S> *__restrict__ C = which ? p1.C : p0.C;
+            const int *__restrict__ ea = which ? p1.ea : p0.ea, *__restrict__ fb = which ? p1.fb : p0.fb;
             const int row = m0 + q * 32 + lane;
             const bool rok = row < M;
             const int cbase = ch * EC;
@@ -601,251 +617,6 @@ oz_update_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
     }
 }
 
-// ---------------------------------------------------------------- slicing
-
-// Balanced base-128 digits of round(v 2^(7 S - e)), v = hi + lo, |v| < 2^(e-1):
-// the scaled value has at most 7 S - 1 bits and the leading digit stays within
-// [-64, 64].  ldexpf scales exactly for any e (the scaled hi is below 2^55; a
-// scaled lo that underflows rounds to 0).
-template <int S> __device__ __forceinline__ void digits(df64 v, int e, int (&d)[S])
-{
-    // Y = rint(hi 2^(S BETA - e)) + rint(lo 2^(S BETA - e)) (|Y| < 2^(7 S - 1)),
-    // written as S balanced base-2^BETA digits, most significant first.  Each
-    // scaled part is an integer-valued float; it is split exactly at
-    // 2^(4 BETA) into two 32-bit integers, so the digits come from 32-bit masks
-    // and shifts: the low four from the low halves (carry into the high half),
-    // the other S - 4 from the high halves.
-    static_assert(S >= 5 && S <= 8 && BETA == 7, "the split at 2^28 leaves at most four digits above it");
-    const float hs = rintf(ldexpf(v.hi, S * BETA - e));
-    const float ls = rintf(ldexpf(v.lo, S * BETA - e));
-    const float hh = rintf(hs * 0x1p-28f), lh = rintf(ls * 0x1p-28f);
-    int low = __float2int_rn(fmaf(-hh, 0x1p28f, hs)) + __float2int_rn(fmaf(-lh, 0x1p28f, ls));  // |low| <= 2^28
-    int high = __float2int_rn(hh) + __float2int_rn(lh);
-#pragma unroll
-    for (int p = S - 1; p >= S - 4; p--) {
-        const int r = ((low & 127) ^ 64) - 64;  // low mod 128, in -64 .. 63
-        d[p] = r;
-        low = (low - r) >> BETA;
-    }
-    high += low;
-#pragma unroll
-    for (int p = S - 5; p >= 1; p--) {
-        const int r = ((high & 127) ^ 64) - 64;
-        d[p] = r;
-        high = (high - r) >> BETA;
-    }
-    d[0] = high;
-}
-
-// Balanced base-128 digits of round(v 2^(63 - e)), |v| < 2^(e-1), v double: the
-// significand shifted to an integer of at most 62 bits (rounded only where
-// bits fall below 2^(e - 63)), its digits from three 32-bit parts (28 bits,
-// 28 bits and the rest) with a carry from each to the next.
-template <int S> __device__ __forceinline__ void digits(double v, int e, int (&d)[S])
-{
-    static_assert(S == kDigits64 && BETA == 7, "two parts of four digits and a leading one");
-    const long long bits = __double_as_longlong(v);
-    const int ex = (int)(bits >> 52) & 0x7FF;
-    const long long m = (bits & 0xFFFFFFFFFFFFFll) | (ex ? 1ll << 52 : 0ll);
-    const int sh = (ex ? ex : 1) - 1075 + S * BETA - e;  // at most 9
-    long long y = sh >= 0 ? m << sh : (sh > -60 ? (m + (1ll << (-sh - 1))) >> -sh : 0ll);
-    if (bits < 0) y = -y;
-    int part[3] = {(int)(y & 0xFFFFFFF), (int)((y >> 28) & 0xFFFFFFF), (int)(y >> 56)};
-#pragma unroll
-    for (int h = 0; h < 2; h++) {
-#pragma unroll
-        for (int p = S - 1 - 4 * h; p >= S - 4 - 4 * h; p--) {
-            const int r = ((part[h] & 127) ^ 64) - 64;  // -64 .. 63
-            d[p] = r;
-            part[h] = (part[h] - r) >> BETA;
-        }
-        part[h + 1] += part[h];
-    }
-    d[0] = part[2];
-}
-
-// A digit (an integer of at most 8 significant bits) as a bf16: it is exact in
-// float (2^23 + 2^22 + r - (2^23 + 2^22) in float arithmetic), and its float's
-// upper half is then the exact bf16.
-__device__ __forceinline__ __nv_bfloat16 bf16_of_digit(int r)
-{
-    const float f = __int_as_float(0x4B400000 + r) - 12582912.0f;
-    return __ushort_as_bfloat16((unsigned short)(__float_as_uint(f) >> 16));
-}
-
-// Binary exponent e of a nonzero float (|x| < 2^e <= 2 |x|); kNoExp for zero.
-// kNoExp is the int whose four bytes are 0x80, so that one memset initializes
-// the atomicMax targets below.
-constexpr int kNoExp = (int)0x80808080u;
-__device__ __forceinline__ int exp_of(float x)
-{
-    if (x == 0.f) return kNoExp;
-    int e;
-    frexpf(x, &e);
-    return e;
-}
-
-__device__ __forceinline__ int exp_of(df64 x) { return exp_of(x.hi); }
-
-// The same for a double (subnormals included); kBadExp for Inf and NaN: a row
-// of A or a column of B that holds one makes its row or column of C NaN, as
-// the products would (an exact zero's product with it is NaN too).
-__device__ __forceinline__ int exp_of(double x)
-{
-    const long long m = __double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFll;
-    const int ex = (int)(m >> 52);
-    if (ex == 0x7FF) return kBadExp;
-    if (m == 0) return kNoExp;
-    return ex ? ex - 1022 : 64 - __clzll(m) - 1074;
-}
-
-__device__ __forceinline__ int finite_exp(int e) { return e == kBadExp ? kNoExp : e; }
-
-// k-balancing exponents, stored as atomicMax targets (initialized to kNoExp):
-// ka[k] = max over rows of E(A_ik), kb[k] = max over columns of E(B_kj).
-// One launch for both: blocks [0, na) take A (block b: column k = b / ca,
-// rows of chunk b % ca, 4096 rows each), the rest take B (64 columns each;
-// threads over k, K <= 512: two per thread at most).
-template <typename TE>
-__global__ void __launch_bounds__(256) kexp_kernel(int M, int K, int N, int ca, int na, const TE *__restrict__ A,
-                                                   int64_t lda, const TE *__restrict__ B, int64_t ldb, int *ka,
-                                                   int *kb)
-{
-    const int b = blockIdx.x;
-    if (b < na) {
-        const int k = b / ca, chunk = b % ca;
-        int e = kNoExp;
-        const int r1 = min(M, (chunk + 1) * 4096);
-        for (int r = chunk * 4096 + threadIdx.x; r < r1; r += 256) e = max(e, finite_exp(exp_of(A[r + (int64_t)k * lda])));
-        for (int o = 16; o > 0; o >>= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
-        if (threadIdx.x % 32 == 0 && e > kNoExp) atomicMax(ka + k, e);
-        return;
-    }
-    const int c0 = (b - na) * 64, c1 = min(N, c0 + 64);
-    for (int k = threadIdx.x; k < K; k += 256) {
-        int e = kNoExp;
-        for (int c = c0; c < c1; c++) e = max(e, finite_exp(exp_of(B[k + (int64_t)c * ldb])));
-        if (e > kNoExp) atomicMax(kb + k, e);
-    }
-}
-
-// t_k of the balancing (0 where column k of A or row k of B is all zero)
-__device__ __forceinline__ int kshift(const int *ka, const int *kb, int k)
-{
-    const int a = ka[k], b = kb[k];
-    if (a == kNoExp || b == kNoExp) return 0;
-    const int d = b - a;
-    return d >= 0 ? d / 2 : -((1 - d) / 2);  // floor(d / 2)
-}
-
-// A (M x K df64, column-major lda) -> S digit slices, slice p at rows p*Mp.. of
-// a K-major [S*Mp][Kp] bf16 array (rows >= M and columns >= K zero), and the
-// row exponents.  32 rows per CTA, 256 threads.  The digit pass goes through
-// a 32 x 32 shared tile: loaded with consecutive threads down a column of A,
-// written with consecutive threads along k of one output row.
-template <int S>
-__device__ __forceinline__ void slice_rows_block(int blk, int M, int K, int Kp, int Mp, const elem_t<S> *__restrict__ A,
-                                                 int64_t lda, const int *__restrict__ ka, const int *__restrict__ kb,
-                                                 __nv_bfloat16 *out, int *ea)
-{
-    __shared__ int smax[32][9];
-    __shared__ int sexp[32];
-    __shared__ elem_t<S> tile[32][33];
-    const int r = threadIdx.x % 32, kl = threadIdx.x / 32;  // 32 rows x 8 lanes of K
-    const int m = blk * 32 + r;
-    int emax = kNoExp;  // max over k of E(A_mk 2^t_k)
-    if (m < M)
-        for (int k = kl; k < K; k += 8) {
-            const int e = exp_of(A[m + (int64_t)k * lda]);
-            if (e != kNoExp) emax = max(emax, e == kBadExp ? e : e + kshift(ka, kb, k));
-        }
-    smax[r][kl] = emax;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        int mx = kNoExp;
-        for (int j = 0; j < 8; j++) mx = max(mx, smax[threadIdx.x][j]);
-        // the pair's low part can push |hi + lo| just past a power of two: one more bit of headroom
-        int e = mx == kNoExp ? 0 : (mx == kBadExp ? mx : mx + 1);
-        sexp[threadIdx.x] = e;
-        int mm = blk * 32 + threadIdx.x;
-        if (mm < M) ea[mm] = e;
-    }
-    const int kk = threadIdx.x % 32, rw = threadIdx.x / 32;  // digit pass: lane = k, warp = row (+ 8 j)
-    for (int k0 = 0; k0 < Kp; k0 += 32) {
-        __syncthreads();  // sexp ready; the previous tile consumed
-#pragma unroll
-        for (int j = 0; j < 4; j++) {
-            const int k = k0 + kl + 8 * j;
-            tile[r][kl + 8 * j] = (m < M && k < K) ? A[m + (int64_t)k * lda] : elem_t<S>(0);
-        }
-        __syncthreads();
-        const int k = k0 + kk;
-#pragma unroll
-        for (int j = 0; j < 4; j++) {
-            const int rr = rw + 8 * j;
-            const int mm = blk * 32 + rr;
-            if (mm >= Mp) continue;
-            int d[S];
-            if (mm < M && k < K && sexp[rr] != kBadExp) {
-                digits<S>(tile[rr][kk], sexp[rr] - kshift(ka, kb, k), d);
-            } else {
-#pragma unroll
-                for (int p = 0; p < S; p++) d[p] = 0;
-            }
-#pragma unroll
-            for (int p = 0; p < S; p++) out[((int64_t)p * Mp + mm) * Kp + k] = bf16_of_digit(d[p]);
-        }
-    }
-}
-
-// B (K x N df64, column-major ldb) -> digit slices of B^T (rows n, K-major), column exponents.
-// One warp per column.
-template <int S>
-__device__ __forceinline__ void slice_cols_warp(int n, int K, int N, int Kp, int Np, const elem_t<S> *__restrict__ B,
-                                                int64_t ldb, const int *__restrict__ ka, const int *__restrict__ kb,
-                                                __nv_bfloat16 *out, int *fb)
-{
-    const int lane = threadIdx.x % 32;
-    if (n >= Np) return;
-    int emax = kNoExp;  // max over k of E(B_kn 2^-t_k)
-    if (n < N)
-        for (int k = lane; k < K; k += 32) {
-            const int e = exp_of(B[k + (int64_t)n * ldb]);
-            if (e != kNoExp) emax = max(emax, e == kBadExp ? e : e - kshift(ka, kb, k));
-        }
-    for (int o = 16; o > 0; o >>= 1) emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, o));
-    const int e = emax == kNoExp ? 0 : (emax == kBadExp ? emax : emax + 1);
-    if (lane == 0 && n < N) fb[n] = e;
-    for (int k = lane; k < Kp; k += 32) {
-        int d[S];
-        if (n < N && k < K && e != kBadExp) {
-            digits<S>(B[k + (int64_t)n * ldb], e + kshift(ka, kb, k), d);
-        } else {
-#pragma unroll
-            for (int p = 0; p < S; p++) d[p] = 0;
-        }
-#pragma unroll
-        for (int p = 0; p < S; p++) out[((int64_t)p * Np + n) * Kp + k] = bf16_of_digit(d[p]);
-    }
-}
-
-// Both slicings in one launch: blocks [0, nra) slice 32 rows of A each, the
-// rest slice 8 columns of B each (one warp per column).
-template <int S>
-__global__ void __launch_bounds__(256, 4) slice_kernel(int M, int N, int K, int Kp, int Mp, int Np, int nra,
-                                                    const elem_t<S> *__restrict__ A, int64_t lda,
-                                                    const elem_t<S> *__restrict__ B, int64_t ldb,
-                                                    const int *__restrict__ ka, const int *__restrict__ kb,
-                                                    __nv_bfloat16 *sa, int *ea, __nv_bfloat16 *sb, int *fb)
-{
-    if ((int)blockIdx.x < nra) {
-        slice_rows_block<S>(blockIdx.x, M, K, Kp, Mp, A, lda, ka, kb, sa, ea);
-    } else {
-        const int n = ((int)blockIdx.x - nra) * 8 + (int)threadIdx.x / 32;
-        slice_cols_warp<S>(n, K, N, Kp, Np, B, ldb, ka, kb, sb, fb);
-    }
-}
-
 __global__ void status_to_info_kernel(const Status *st, int64_t *info)
 {
     if (st->err != 0 && *info < 0) *info = -2;
@@ -898,9 +669,11 @@ namespace oz {
 
 template <int S> static rbt_status configure()
 {
-    static PerDeviceOnce once;
-    static PerDeviceOnce once_raw;
+    static PerDeviceOnce once, once_raw, once_out, once_wide;
     rbt_status st = smem_opt_in(once, oz_update_kernel<false, S>, kSmemBytes<S>);
+    if (st == RBT_OK) st = smem_opt_in(once_out, slice_kernel<S, 32, false>, (int)slice_smem_bytes<S>(KMAX<S>));
+    if (st == RBT_OK && kWide<S>)
+        st = smem_opt_in(once_wide, slice_kernel<S, 32, kWide<S>>, (int)slice_smem_bytes<S>(kOuterNB<S>));
     if (st != RBT_OK || S != 8) return st;
     return smem_opt_in(once_raw, oz_update_kernel<true, 8>, kSmemBytes<8>);
 }
@@ -911,6 +684,7 @@ struct Slices {
     __nv_bfloat16 *sa, *sb;
     int *ea, *fb, *ka, *kb;
     int64_t M, N, K, Mp, Np, Kp;
+    char *end;
 };
 
 template <int S> static Slices carve(int64_t M, int64_t N, int64_t K, void *work)
@@ -934,65 +708,92 @@ template <int S> static Slices carve(int64_t M, int64_t N, int64_t K, void *work
     sl.ka = (int *)w;
     w += rup(sl.Kp * 4, 256);
     sl.kb = (int *)w;
+    w += rup(sl.Kp * 4, 256);
+    sl.end = (char *)work + rup(w - (char *)work, 1024);
     return sl;
 }
 
-// The balancing exponents and digit slices of A (M x K) and B (K x N).
-template <int S>
-static rbt_status slice(const Slices &sl, const elem_t<S> *A, int64_t lda, const elem_t<S> *B, int64_t ldb,
-                        cudaStream_t stream)
-{
-    const int64_t M = sl.M, N = sl.N, K = sl.K;
-    if (M <= 0 || N <= 0 || K <= 0) return RBT_OK;
-    ProfScope pslice(kProfSlice, stream);
-    // both exponent arrays start at kNoExp (every byte 0x80)
-    RBT_CUDA_TRY(cudaMemsetAsync(sl.ka, 0x80, (size_t)rup(sl.Kp * 4, 256) * 2, stream));
-    const int ca = (int)cdiv(M, 4096), na = ca * (int)K;
-    kexp_kernel<elem_t<S>><<<(unsigned)(na + cdiv(N, 64)), 256, 0, stream>>>((int)M, (int)K, (int)N, ca, na, A, lda, B, ldb,
-                                                                    sl.ka, sl.kb);
-    RBT_LAUNCH_CHECK();
-    const int nra = (int)cdiv(sl.Mp, 32);
-    slice_kernel<S><<<(unsigned)(nra + cdiv(sl.Np, 8)), 256, 0, stream>>>(
-        (int)M, (int)N, (int)K, (int)sl.Kp, (int)sl.Mp, (int)sl.Np, nra, A, lda, B, ldb, sl.ka, sl.kb, sl.sa, sl.ea,
-        sl.sb, sl.fb);
-    RBT_LAUNCH_CHECK();
-    return RBT_OK;
-}
+// The operands of one product C (M x N) -= A B and the balancing exponents of
+// its K (ka and ka2: of A's columns, the larger counts; kb: of B's rows).
+template <int S> struct Operands {
+    int64_t M, N;
+    const elem_t<S> *A, *B;
+    elem_t<S> *C;
+    const int *ka, *ka2, *kb;
+};
 
-// C (Ms x Ns, ldc) -= rows [a0, a0 + Ms) of A times columns [b0, b0 + Ns) of
-// B from the slices (a0 a multiple of BM, b0 of BN, both blocks inside the
-// sliced product), on at most max_ctas CTAs.
-template <int S>
-static rbt_status multiply(const Slices &sl, int64_t a0, int64_t b0, int64_t Ms, int64_t Ns, elem_t<S> *C, int64_t ldc,
-                           const int64_t *info, void *status, unsigned max_ctas, cudaStream_t stream)
+// One or two products of the same K and leading dimensions: the digit slices
+// of all operands in one launch, the products in another.
+template <int S, bool WIDE>
+static rbt_status products(int count, const Operands<S> *op, const Slices *sl, int64_t K, int64_t lda, int64_t ldb,
+                           int64_t ldc, const int64_t *info, void *status, unsigned max_ctas, cudaStream_t stream)
 {
-    if (Ms <= 0 || Ns <= 0) return RBT_OK;
-    if (a0 % BM || b0 % BN<S> || a0 < 0 || b0 < 0 || a0 + Ms > sl.M || b0 + Ns > sl.N) return RBT_ERR_ARG;
+    using TE = elem_t<S>;
+    const int Kp = (int)rup(K, KSLAB);
+    {
+        ProfScope pslice(kProfSlice, stream);
+        SliceJobs<TE> jobs = {};
+        const int per = K <= 64 ? 16 : 8;  // columns of B per CTA
+        int64_t blocks = 0;
+        for (int i = 0; i < count; i++) {
+            const int nra = (int)(sl[i].Mp / kSliceRows), nrb = (int)cdiv(sl[i].Np, per);
+            jobs.job[2 * i] = {op[i].A, lda, (int)op[i].M, (int)sl[i].Mp, op[i].ka, op[i].ka2, op[i].kb,
+                               sl[i].sa, sl[i].ea, 1, nra};
+            jobs.job[2 * i + 1] = {op[i].B, ldb, (int)op[i].N, (int)sl[i].Np, op[i].ka, op[i].ka2, op[i].kb,
+                                   sl[i].sb, sl[i].fb, 0, nrb};
+            blocks += nra + nrb;
+        }
+        jobs.K = (int)K;
+        jobs.Kp = Kp;
+        if (K <= 64)
+            slice_kernel<S, 16, WIDE><<<(unsigned)blocks, 256, slice_smem_bytes<S>(Kp), stream>>>(jobs);
+        else
+            slice_kernel<S, 32, WIDE><<<(unsigned)blocks, 256, slice_smem_bytes<S>(Kp), stream>>>(jobs);
+        RBT_LAUNCH_CHECK();
+    }
     ProfScope ps(kProfUpdate, stream);
-    CUtensorMap ma, mb;
-    if (!make_map(&ma, sl.sa, (int)(S * sl.Mp), (int)sl.Kp, BM) || !make_map(&mb, sl.sb, (int)(S * sl.Np), (int)sl.Kp, BN<S>))
-        return RBT_ERR_CUDA;
-    const int64_t ntiles = cdiv(Ms, BM) * cdiv(Ns, BN<S>);
-    const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(ntiles, max_ctas));
+    CUtensorMap ma[2], mb[2];
+    Problem<S> p[2] = {};
+    for (int i = 0; i < count; i++) {
+        if (!make_map(&ma[i], sl[i].sa, (int)(S * sl[i].Mp), Kp, BM) ||
+            !make_map(&mb[i], sl[i].sb, (int)(S * sl[i].Np), Kp, BN<S>))
+            return RBT_ERR_CUDA;
+        const int tm = (int)cdiv(op[i].M, BM), tn = (int)cdiv(op[i].N, BN<S>);
+        p[i] = {(int)op[i].M, (int)op[i].N, (int)sl[i].Mp, (int)sl[i].Np, sl[i].ea, sl[i].fb, op[i].C, ldc, tm, tn,
+                (int64_t)tm * tn};
+    }
+    if (count < 2) {
+        ma[1] = ma[0];
+        mb[1] = mb[0];
+    }
+    const unsigned grid = (unsigned)std::min<int64_t>(p[0].ntiles + p[1].ntiles, max_ctas);
     oz_update_kernel<false, S><<<grid, kOzThreads, kSmemBytes<S>, stream>>>(
-        ma, mb, (int)Ms, (int)Ns, (int)sl.Kp, (int)sl.Mp, (int)sl.Np, (int)a0, (int)b0, sl.ea + a0, sl.fb + b0, C,
-        ldc, info, (Status *)status, wait_limit_ns(), debug_stall() == RBT_STALL_OZ_COPY ? 1 : 0, nullptr);
+        ma[0], mb[0], ma[1], mb[1], p[0], p[1], Kp, info, (Status *)status, wait_limit_ns(),
+        debug_stall() == RBT_STALL_OZ_COPY ? 1 : 0, nullptr);
     RBT_LAUNCH_CHECK();
     return RBT_OK;
 }
 
+// A standalone update: its balancing exponents come from a pass of their own.
 template <int S>
 static rbt_status update(int64_t M, int64_t N, int64_t K, const elem_t<S> *A, int64_t lda, const elem_t<S> *B,
-                         int64_t ldb, elem_t<S> *C, int64_t ldc, const int64_t *info, void *work, void *status, unsigned max_ctas,
-                         cudaStream_t stream)
+                         int64_t ldb, elem_t<S> *C, int64_t ldc, const int64_t *info, void *work, void *status,
+                         unsigned max_ctas, cudaStream_t stream)
 {
-    if (M <= 0 || N <= 0 || K <= 0) return RBT_OK;
     rbt_status s = configure<S>();
     if (s != RBT_OK) return s;
     const Slices sl = carve<S>(M, N, K, work);
-    s = slice<S>(sl, A, lda, B, ldb, stream);
-    if (s != RBT_OK) return s;
-    return multiply<S>(sl, 0, 0, M, N, C, ldc, info, status, max_ctas, stream);
+    {
+        ProfScope pslice(kProfSlice, stream);
+        // both exponent arrays start at kNoExp (every byte 0x80)
+        RBT_CUDA_TRY(cudaMemsetAsync(sl.ka, 0x80, (size_t)rup(sl.Kp * 4, 256) * 2, stream));
+        const int ca = (int)cdiv(M, 4096), na = ca * (int)K;
+        kexp_kernel<elem_t<S>><<<(unsigned)(na + cdiv(N, 64)), 256, 0, stream>>>((int)M, (int)K, (int)N, ca, na, A, lda,
+                                                                              B, ldb, sl.ka, sl.kb);
+        RBT_LAUNCH_CHECK();
+    }
+    const Operands<S> op = {M, N, A, B, C, sl.ka, sl.ka, sl.kb};
+    return products<S, false>(1, &op, &sl, K, lda, ldb, ldc, info, status, max_ctas, stream);
 }
 
 }  // namespace oz
@@ -1083,9 +884,10 @@ rbt_status oz_products(int64_t M, int64_t N, int64_t K, const int8_t *da, const 
         return RBT_ERR_CUDA;
     const int64_t ntiles = (Mp / BM) * (Np / BN<kRawDigits>);
     const unsigned grid = (unsigned)std::min<int64_t>(ntiles, device_sm_count());
-    oz_update_kernel<true, kRawDigits><<<grid, kOzThreads, kSmemBytes<kRawDigits>, stream>>>(ma, mb, (int)M, (int)N, (int)Kp, (int)Mp,
-                                                                     (int)Np, 0, 0, nullptr, nullptr, nullptr, 0, info,
-                                                                     status, wait_limit_ns(), 0, acc);
+    const int tm = (int)(Mp / BM), tn = (int)(Np / BN<kRawDigits>);
+    const Problem<kRawDigits> p = {(int)M, (int)N, (int)Mp, (int)Np, nullptr, nullptr, nullptr, 0, tm, tn, ntiles}, none = {};
+    oz_update_kernel<true, kRawDigits><<<grid, kOzThreads, kSmemBytes<kRawDigits>, stream>>>(
+        ma, mb, ma, mb, p, none, (int)Kp, info, status, wait_limit_ns(), 0, acc);
     RBT_LAUNCH_CHECK();
     return RBT_OK;
 }
@@ -1109,49 +911,65 @@ rbt_status rbt_debug_oz_products(int64_t M, int64_t N, int64_t K, const int8_t *
 
 namespace rbt {
 
-// K of the trailing update: the digit-product exactness bound
 constexpr int kOzInnerNB = 64;   // panel step (double-float diagonal factor and TRSMs)
 
 size_t oz_factor_workspace(int64_t n)
 {
     if (n <= 0) return 0;
-    // any digit count
-    return std::max(oz_update_workspace(n, n, oz::KMAX<8>, 8), oz_update_workspace(n, n, oz::KMAX<9>, 9)) + 256;
+    // any digit count: an outer update's slices (far more than the two inner
+    // ones'), the balancing exponents of a panel, the status word
+    return std::max(oz_update_workspace(n, n, oz::KMAX<8>, 8), oz_update_workspace(n, n, oz::KMAX<9>, 9)) + 16384 +
+           4 * kKmax * sizeof(int) + 256;
 }
 
 namespace {
 
-// Two-level blocked GENP in double-float: panels of 512 columns factored with
-// 64-column steps (shared-memory diagonal factor and both TRSMs in
-// double-float, sliced tensor-core updates of the panel and of the row block
-// to its right), then one rank-512 sliced tensor-core update of the trailing
-// matrix per panel.
+// Two-level blocked GENP: panels of 512 columns (448 with seven digits and in
+// double) factored with
+// 64-column steps (diagonal factor and both TRSMs on the SIMT pipes, one
+// launch of sliced tensor-core updates of the panel's remaining columns and of
+// the rest of its rows), then one sliced update of the trailing matrix per
+// panel.  The TRSMs leave the exponents that balance every update (per column
+// of L21 and row of U12, split at the panel's end), so an update is two
+// launches: slicing and products.
 template <int S>
 rbt_status factor_oz(int64_t n, oz::elem_t<S> *A, int64_t lda, int64_t *info, void *work, cudaStream_t stream)
 {
-    constexpr int kOzOuterNB = oz::KMAX<S>;
-    const size_t ws = oz_factor_workspace(n) - 256;
-    void *status = (char *)work + ws;
+    constexpr int kOuter = oz::kOuterNB<S>;
+    rbt_status s = oz::configure<S>();
+    if (s != RBT_OK) return s;
+    void *status = (char *)work + oz_factor_workspace(n) - 256;
+    int *kmax = (int *)status - 4 * kKmax;
+    int *rows_in = kmax, *rows_below = kmax + kKmax, *cols_in = kmax + 2 * kKmax, *cols_right = kmax + 3 * kKmax;
     RBT_CUDA_TRY(cudaMemsetAsync(status, 0, 256, stream));
     const unsigned sms = (unsigned)device_sm_count();
-    rbt_status s;
-    for (int64_t k = 0; k < n; k += kOzOuterNB) {
-        const int64_t kb = n - k < kOzOuterNB ? n - k : kOzOuterNB;
-        for (int64_t j = k; j < k + kb; j += kOzInnerNB) {
-            const int jb = (int)(k + kb - j < kOzInnerNB ? k + kb - j : kOzInnerNB);
-            s = genp_panel_steps<oz::elem_t<S>>(n, A, lda, info, jb, j, j + jb, false, stream);
+    for (int64_t k = 0; k < n; k += kOuter) {
+        const int64_t kb = n - k < kOuter ? n - k : kOuter;
+        const int64_t t0 = k + kb, right = n - t0;
+        if (n - k > kOzInnerNB)
+            RBT_CUDA_TRY(cudaMemsetAsync(kmax, 0x80, 4 * kKmax * sizeof(int), stream));  // kNoExp
+        for (int64_t j = k; j < t0; j += kOzInnerNB) {
+            const int jb = (int)(t0 - j < kOzInnerNB ? t0 - j : kOzInnerNB);
+            const int64_t r0 = j + jb, at = j - k;
+            s = genp_panel_steps<oz::elem_t<S>>(n, A, lda, info, jb, j, r0, false, stream, t0, kmax + at);
             if (s != RBT_OK) return s;
-            const int64_t r0 = j + jb;
-            s = oz::update<S>(n - r0, k + kb - r0, jb, A + r0 + j * lda, lda, A + j + r0 * lda, lda,
-                              A + r0 + r0 * lda, lda, info, work, status, sms, stream);
-            if (s != RBT_OK) return s;
-            s = oz::update<S>(k + kb - r0, n - k - kb, jb, A + r0 + j * lda, lda, A + j + (k + kb) * lda, lda,
-                              A + r0 + (k + kb) * lda, lda, info, work, status, sms, stream);
+            if (r0 >= t0) continue;
+            const oz::Operands<S> op[2] = {
+                {n - r0, t0 - r0, A + r0 + j * lda, A + j + r0 * lda, A + r0 + r0 * lda, rows_in + at, rows_below + at,
+                 cols_in + at},
+                {t0 - r0, right, A + r0 + j * lda, A + j + t0 * lda, A + r0 + t0 * lda, rows_in + at, rows_in + at,
+                 cols_right + at}};
+            oz::Slices sl[2];
+            sl[0] = oz::carve<S>(op[0].M, op[0].N, jb, work);
+            sl[1] = oz::carve<S>(op[1].M, op[1].N, jb, sl[0].end);
+            s = oz::products<S, oz::kWide<S>>(right > 0 ? 2 : 1, op, sl, jb, lda, lda, lda, info, status, sms, stream);
             if (s != RBT_OK) return s;
         }
-        const int64_t t0 = k + kb;
-        s = oz::update<S>(n - t0, n - t0, kb, A + t0 + k * lda, lda, A + k + t0 * lda, lda, A + t0 + t0 * lda, lda,
-                          info, work, status, sms, stream);
+        if (right <= 0) continue;
+        const oz::Operands<S> op = {right, right, A + t0 + k * lda, A + k + t0 * lda, A + t0 + t0 * lda, rows_below,
+                                    rows_below, cols_right};
+        const oz::Slices sl = oz::carve<S>(right, right, kb, work);
+        s = oz::products<S, oz::kWide<S>>(1, &op, &sl, kb, lda, lda, lda, info, status, sms, stream);
         if (s != RBT_OK) return s;
     }
     return oz_status_to_info(status, info, stream);

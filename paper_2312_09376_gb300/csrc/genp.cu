@@ -19,6 +19,7 @@
 #include "common.cuh"
 #include "genp_internal.cuh"
 #include "df64.cuh"
+#include "oz_slice.cuh"
 
 #include <type_traits>
 
@@ -201,6 +202,342 @@ __global__ void __launch_bounds__(kTrsmThreads) trsm_panel_kernel(int64_t k0, in
             if (row < n) A[row + (k0 + j) * lda] = X[j * kTrsmXS + r];
         }
     }
+}
+
+// ------------------------------------------- blocks of at most 64 columns
+//
+// A multiply-subtract of the elimination.  In double-float the sum is
+// renormalized but not the product (15 operations instead of 19);
+// renormalizing only every fourth one (12) makes unrefined backward errors two
+// to three times larger.
+constexpr int kP = 64;  // columns of a block
+constexpr int kQ = 16;  // columns of a panel inside it
+
+template <typename T> __device__ __forceinline__ void sub_mul(T &a, T c, T x) { a = fma(-c, x, a); }
+template <> __device__ __forceinline__ void sub_mul<df64>(df64 &a, df64 c, df64 x)
+{
+    const float p = __fmul_rn(-c.hi, x.hi);
+    const float pe = __fmaf_rn(-c.hi, x.hi, -p);
+    float s, e;
+    two_sum(a.hi, p, s, e);
+    a = df_norm(s, __fadd_rn(e, __fadd_rn(a.lo, __fmaf_rn(-c.lo, x.hi, __fmaf_rn(-c.hi, x.lo, pe)))));
+}
+
+// N independent ones, a[i] -= c[i] x, written stage by stage: each stage's
+// operations are independent, where one entry after the other leaves the
+// instruction order a single dependent chain.
+template <int N, typename T> __device__ __forceinline__ void sub_mul_n(T (&a)[N], const T (&c)[N], T x)
+{
+#pragma unroll
+    for (int i = 0; i < N; i++) a[i] = fma(-c[i], x, a[i]);
+}
+template <int N> __device__ __forceinline__ void sub_mul_n(df64 (&a)[N], const df64 (&c)[N], df64 x)
+{
+    float p[N], l[N], s[N], b[N], u[N];
+#pragma unroll
+    for (int i = 0; i < N; i++) p[i] = __fmul_rn(-c[i].hi, x.hi);
+#pragma unroll
+    for (int i = 0; i < N; i++) l[i] = __fmaf_rn(-c[i].hi, x.hi, -p[i]);
+#pragma unroll
+    for (int i = 0; i < N; i++) s[i] = __fadd_rn(a[i].hi, p[i]);
+#pragma unroll
+    for (int i = 0; i < N; i++) l[i] = __fmaf_rn(-c[i].hi, x.lo, l[i]);
+#pragma unroll
+    for (int i = 0; i < N; i++) b[i] = __fsub_rn(s[i], a[i].hi);
+#pragma unroll
+    for (int i = 0; i < N; i++) l[i] = __fmaf_rn(-c[i].lo, x.hi, l[i]);
+#pragma unroll
+    for (int i = 0; i < N; i++) u[i] = __fsub_rn(s[i], b[i]);
+#pragma unroll
+    for (int i = 0; i < N; i++) p[i] = __fsub_rn(p[i], b[i]);
+#pragma unroll
+    for (int i = 0; i < N; i++) u[i] = __fsub_rn(a[i].hi, u[i]);
+#pragma unroll
+    for (int i = 0; i < N; i++) l[i] = __fadd_rn(a[i].lo, l[i]);
+#pragma unroll
+    for (int i = 0; i < N; i++) u[i] = __fadd_rn(u[i], p[i]);
+#pragma unroll
+    for (int i = 0; i < N; i++) l[i] = __fadd_rn(u[i], l[i]);
+#pragma unroll
+    for (int i = 0; i < N; i++) a[i].hi = __fadd_rn(s[i], l[i]);
+#pragma unroll
+    for (int i = 0; i < N; i++) s[i] = __fsub_rn(a[i].hi, s[i]);
+#pragma unroll
+    for (int i = 0; i < N; i++) a[i].lo = __fsub_rn(l[i], s[i]);
+}
+
+// a / p from r, an approximate reciprocal of p (of its leading part in
+// double-float): the quotient's residual is taken once more (as in a division
+// by Newton's iteration), so a step costs one reciprocal and the quotients a
+// few multiply-adds each, at the accuracy of the division.  Pivots near the
+// ends of the exponent range take the division itself.
+__device__ __forceinline__ bool mid_range(double p) { return fabs(p) > 1e-30 && fabs(p) < 1e30; }
+__device__ __forceinline__ bool mid_range(float p) { return fabsf(p) > 1e-30f && fabsf(p) < 1e30f; }
+__device__ __forceinline__ bool mid_range(df64 p) { return mid_range(p.hi); }
+template <typename T> __device__ __forceinline__ T recip(T p);
+template <> __device__ __forceinline__ float recip<float>(float p) { return __frcp_rn(p); }
+template <> __device__ __forceinline__ df64 recip<df64>(df64 p) { return df64(__frcp_rn(p.hi)); }
+// a float's reciprocal and one Newton step (2^-46): the FP64 pipe's operations
+// are the chain's long ones, and the quotient's residual step follows anyway
+template <> __device__ __forceinline__ double recip<double>(double p)
+{
+    const double r = (double)__frcp_rn((float)p);
+    return ::fma(r, ::fma(-p, r, 1.0), r);
+}
+template <typename T> __device__ __forceinline__ T quotient(T a, T p, T r, bool mid)
+{
+    if (!mid) return a / p;
+    const T l = a * r;
+    return fma(fma(-l, p, a), r, l);
+}
+template <> __device__ __forceinline__ df64 quotient<df64>(df64 a, df64 p, df64 r, bool mid)
+{
+    if (!mid) return a / p;
+    const float q = __fmul_rn(a.hi, r.hi);
+    const float t = __fmaf_rn(-q, p.hi, a.hi);  // exact: q p.hi agrees with a.hi to a few units
+    const float d = __fmaf_rn(-q, p.lo, __fadd_rn(t, a.lo));
+    return df_norm(q, __fmul_rn(d, r.hi));
+}
+
+// Diagonal block (kb <= 64): one CTA, four lanes per row, in panels of 16
+// columns.  Inside a panel a step is the pivot row's at most 16 entries
+// published through shared memory with the pivot's reciprocal, one barrier, a
+// quotient and at most four multiply-subtracts a lane: the chain of 64 steps
+// is what the kernel costs, so nothing else is on it.  Then the panel's rows
+// of the columns to the right (a 16-step substitution, four lanes a column)
+// and the rank-16 update of the rest (up to 12 independent entries a lane).
+template <typename T>
+__global__ void __launch_bounds__(256, 1) diag64_kernel(int64_t k0, int kb, T *A, int64_t lda, int64_t *info)
+{
+    constexpr int LD = kP + 1;
+    __shared__ T S[kP * LD];  // the block, row-major
+    __shared__ T urow[2][kQ];
+    __shared__ T piv[2][2];
+    if (info_set(info)) return;
+    const int tid = threadIdx.x, i = tid / 4, q = tid % 4, gbase = tid & 28;
+    for (int e = tid; e < kP * kP; e += 256) {
+        const int r = e % kP, c = e / kP;
+        S[r * LD + c] = (r < kb && c < kb) ? A[(k0 + r) + (k0 + c) * lda] : T(0);
+    }
+    __syncthreads();
+    bool stop = false;
+    for (int c0 = 0; c0 < kb && !stop; c0 += kQ) {
+        T a[4];
+#pragma unroll
+        for (int r = 0; r < 4; r++) a[r] = S[i * LD + c0 + q + 4 * r];
+#pragma unroll
+        for (int jj = 0; jj < kQ; jj++) {
+            const int j = c0 + jj;
+            if (stop || j >= kb) continue;  // the same in every thread
+            T *u = urow[jj & 1], *pv = piv[jj & 1];
+            if (i == j) {
+                if (q == jj % 4) {
+                    pv[0] = a[jj / 4];
+                    pv[1] = recip(a[jj / 4]);
+                }
+#pragma unroll
+                for (int r = jj / 4; r < 4; r++) u[q + 4 * r] = a[r];
+            }
+            __syncthreads();
+            const T p = pv[0];
+            if (bad_pivot(p)) {  // every thread reads the same pivot: a uniform exit
+                if (tid == 0) *info = k0 + j;
+                stop = true;
+                continue;
+            }
+            if ((i | 7) > j) {  // some row of the warp is below the pivot
+                const T l = quotient(shfl_idx(a[jj / 4], gbase | (jj % 4)), p, pv[1], mid_range(p));
+                if (i > j) {
+                    T w[4], v[4];
+#pragma unroll
+                    for (int r = 0; r < 4; r++) {
+                        w[r] = a[r];
+                        v[r] = u[q + 4 * r];
+                    }
+                    sub_mul_n(w, v, l);
+                    if (q > jj % 4) a[jj / 4] = w[jj / 4];
+                    if (q == jj % 4) a[jj / 4] = l;
+#pragma unroll
+                    for (int r = jj / 4 + 1; r < 4; r++) a[r] = w[r];
+                }
+            }
+        }
+        if (i >= c0)
+#pragma unroll
+            for (int r = 0; r < 4; r++) S[i * LD + c0 + q + 4 * r] = a[r];
+        __syncthreads();
+        const int c1 = c0 + kQ;
+        if (c1 >= kb || stop) continue;
+        // rows c0 .. c1 - 1 of the columns right of the panel
+        if (i < kP - c1) {
+            const int c = c1 + i;
+#pragma unroll
+            for (int r = 0; r < 4; r++) a[r] = S[(c0 + q + 4 * r) * LD + c];
+#pragma unroll
+            for (int jj = 0; jj < kQ; jj++) {
+                const T x = shfl_idx(a[jj / 4], gbase | (jj % 4));
+                T w[4], l[4];
+#pragma unroll
+                for (int r = 0; r < 4; r++) {
+                    w[r] = a[r];
+                    l[r] = S[(c0 + q + 4 * r) * LD + c0 + jj];
+                }
+                sub_mul_n(w, l, x);
+                if (q > jj % 4) a[jj / 4] = w[jj / 4];
+#pragma unroll
+                for (int r = jj / 4 + 1; r < 4; r++) a[r] = w[r];
+            }
+#pragma unroll
+            for (int r = 0; r < 4; r++) S[(c0 + q + 4 * r) * LD + c] = a[r];
+        }
+        __syncthreads();
+        // the rest: rows and columns from c1 on
+        if (i >= c1) {
+            const int nc = (kP - c1) / 4;  // 12, 8 or 4 columns a lane
+            for (int g = 0; g < nc; g += 4) {
+                const int cg = c1 + q + 4 * g;
+                T w[4], u[4];
+#pragma unroll
+                for (int r = 0; r < 4; r++) w[r] = S[i * LD + cg + 4 * r];
+#pragma unroll 4
+                for (int k = 0; k < kQ; k++) {
+#pragma unroll
+                    for (int r = 0; r < 4; r++) u[r] = S[(c0 + k) * LD + cg + 4 * r];
+                    sub_mul_n(w, u, S[i * LD + c0 + k]);
+                }
+#pragma unroll
+                for (int r = 0; r < 4; r++) S[i * LD + cg + 4 * r] = w[r];
+            }
+        }
+        __syncthreads();
+    }
+    __syncthreads();
+    // write back (the partial factor too when stopped: the caller ignores it)
+    for (int e = tid; e < kP * kP; e += 256) {
+        const int r = e % kP, c = e / kP;
+        if (r < kb && c < kb) A[(k0 + r) + (k0 + c) * lda] = S[r * LD + c];
+    }
+}
+
+// Both TRSMs of a step, U12 <- L11^{-1} A12 (blocks [0, nbu), a vector is a
+// column) and L21 <- A21 U11^{-1} (the other blocks, a vector is a row): the
+// substitution runs right-looking down each vector, VEC vectors per CTA on
+// LANES lanes each (lane q holds the entries q + LANES r in registers), the
+// block's coefficients in shared memory.  Each thread carries NV vectors, so
+// that a coefficient read serves NV multiply-subtracts (with one, the
+// shared-memory reads bound the double-float kernel).  The loop runs LANES
+// steps at a time and then moves each lane's entries down by one register,
+// which makes the finished ones a[0] (a fixed register) without unrolling all
+// 64 steps; entries past the block's end are skipped four at a time (a test of
+// each would leave no independent instructions to interleave).  Entries come
+// and go without staging.  kmax, when given, receives the exponents that
+// balance the sliced updates (gemm_oz.cu): for each k the largest over the
+// panel's own rows, the rows below it, its columns, and the columns right of
+// it, each in an array of kKmax ints.
+template <typename T, int VEC, int LANES, int NV>
+__global__ void __launch_bounds__(VEC * LANES / NV)
+trsm64_kernel(int64_t k0, int kb, int64_t n, T *A, int64_t lda, int nbu, const int64_t *info, int64_t panel_end,
+              int *kmax)
+{
+    constexpr int E = kP / LANES, NT = VEC * LANES / NV;
+    // M(k, j), the entry that couples j into k, at k + 65 j (past the last
+    // column: read with the last entries' groups, never used)
+    __shared__ T Mt[kP * (kP + 1) + kP];
+    __shared__ T rd[kP];
+    __shared__ int kx[kP];
+    if (info_set(info)) return;
+    const int tid = threadIdx.x, q = tid % LANES, gbase = tid & 31 & ~(LANES - 1);
+    const bool upper = (int)blockIdx.x < nbu;
+    const int64_t first = k0 + kb + (int64_t)(upper ? blockIdx.x : blockIdx.x - nbu) * VEC;
+    const int64_t es = upper ? 1 : lda;
+    T a[NV][E];
+    T *base[NV];  // entry e at base[e * es]
+    bool in[NV];
+#pragma unroll
+    for (int w = 0; w < NV; w++) {
+        const int64_t v = first + tid / LANES + w * (VEC / NV);
+        in[w] = v < n;
+        base[w] = upper ? A + k0 + v * lda : A + v + k0 * lda;
+#pragma unroll
+        for (int r = 0; r < E; r++)
+            a[w][r] = (in[w] && q + LANES * r < kb) ? base[w][(q + LANES * r) * es] : T(0);
+    }
+    for (int e = tid; e < kP * kP; e += NT) {
+        const int i = e % kP, j = e / kP;
+        const T m = (i < kb && j < kb) ? A[(k0 + i) + (k0 + j) * lda] : T(0);
+        Mt[upper ? i + j * (kP + 1) : j + i * (kP + 1)] = m;
+    }
+    for (int j = tid; j < kP; j += NT) {
+        rd[j] = (j < kb && !upper) ? T(1) / A[(k0 + j) + (k0 + j) * lda] : T(1);
+        kx[j] = kNoExp;
+    }
+    __syncthreads();
+    for (int jb = 0; LANES * jb < kb; jb++) {
+#pragma unroll
+        for (int jj = 0; jj < LANES; jj++) {
+            const int j = LANES * jb + jj;
+            const T *m = Mt + j * (kP + 1) + q + LANES * jb;
+            T x[NV];
+#pragma unroll
+            for (int w = 0; w < NV; w++) {
+                if (q == jj && !upper) a[w][0] = a[w][0] * rd[j];
+                x[w] = shfl_idx(a[w][0], gbase | jj);
+                if (q > jj) sub_mul(a[w][0], m[0], x[w]);
+            }
+#pragma unroll
+            for (int g = 1; g < E; g += 4)
+                if (jb + g < E) {
+                    constexpr int G = 4;
+                    T c[G];
+#pragma unroll
+                    for (int r = 0; r < G; r++) c[r] = g + r < E ? m[LANES * (g + r)] : T(0);
+#pragma unroll
+                    for (int w = 0; w < NV; w++) {
+                        T v[G];
+#pragma unroll
+                        for (int r = 0; r < G; r++) v[r] = g + r < E ? a[w][g + r] : T(0);
+                        sub_mul_n(v, c, x[w]);
+#pragma unroll
+                        for (int r = 0; r < G; r++)
+                            if (g + r < E) a[w][g + r] = v[r];
+                    }
+                }
+        }
+        const int c = q + LANES * jb;
+        int e = kNoExp;
+#pragma unroll
+        for (int w = 0; w < NV; w++)
+            if (in[w] && c < kb) {
+                base[w][c * es] = a[w][0];
+                e = max(e, finite_exp(exp_of(a[w][0])));
+            }
+        if (kmax) {
+#pragma unroll
+            for (int o = LANES; o < 32; o <<= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
+            if ((tid & 31) < LANES && e > kNoExp) atomicMax(kx + c, e);
+        }
+#pragma unroll
+        for (int w = 0; w < NV; w++)
+#pragma unroll
+            for (int r = 0; r + 1 < E; r++) a[w][r] = a[w][r + 1];
+    }
+    if (kmax) {
+        __syncthreads();
+        // first is at a distance from k0 + kb that VEC divides, and the panel's
+        // end at one that 64 divides: a CTA's vectors lie on one side of it
+        int *to = kmax + (upper ? 2 : 0) * kKmax + (first < panel_end ? 0 : kKmax);
+        for (int j = tid; j < kb; j += NT)
+            if (kx[j] > kNoExp) atomicMax(to + j, kx[j]);
+    }
+}
+
+template <typename T, int VEC, int LANES, int NV>
+static void launch_trsm64(int64_t k, int kb, int64_t n, T *A, int64_t lda, const int64_t *info, int64_t panel_end,
+                          int *kmax, cudaStream_t stream)
+{
+    const int nbv = (int)cdiv(n - k - kb, VEC);
+    trsm64_kernel<T, VEC, LANES, NV><<<(unsigned)(2 * nbv), VEC * LANES / NV, 0, stream>>>(k, kb, n, A, lda, nbv, info,
+                                                                                          panel_end, kmax);
 }
 
 // ------------------------------------------------------------- SIMT GEMM
@@ -551,20 +888,33 @@ template rbt_status gemm_sub_simt<df64>(int64_t, int64_t, int, const df64 *, int
 
 template <typename T>
 rbt_status genp_panel_steps(int64_t n, T *A, int64_t lda, int64_t *info, int nb, int64_t k0, int64_t k_end,
-                            bool trailing_simt, cudaStream_t stream)
+                            bool trailing_simt, cudaStream_t stream, int64_t panel_end, int *kmax)
 {
     for (int64_t k = k0; k < k_end; k += nb) {
         int kb = (int)(n - k < nb ? n - k : nb);
         int64_t rest = n - k - kb;
         {
             ProfScope ps(kProfPanel, stream);
-            size_t sm = (size_t)kb * kb * sizeof(T);
-            diag_factor_kernel<T><<<1, 256, sm, stream>>>(k, kb, A, lda, info);
+            if (kb <= kP) {
+                diag64_kernel<T><<<1, 256, 0, stream>>>(k, kb, A, lda, info);
+            } else {
+                size_t sm = (size_t)kb * kb * sizeof(T);
+                diag_factor_kernel<T><<<1, 256, sm, stream>>>(k, kb, A, lda, info);
+            }
             RBT_LAUNCH_CHECK();
             if (rest <= 0) continue;
-            size_t sm_t = trsm_smem_bytes<T>(kb);
-            const int nbv = (int)cdiv(rest, kTrsmVec);
-            trsm_panel_kernel<T><<<(unsigned)(2 * nbv), kTrsmThreads, sm_t, stream>>>(k, kb, n, A, lda, nbv, info);
+            if (kb <= kP) {
+                if constexpr (std::is_same<T, double>::value)
+                    launch_trsm64<T, 8, 16, 1>(k, kb, n, A, lda, info, panel_end, kmax, stream);
+                else if (2 * cdiv(rest, 64) >= kNumSMs)
+                    launch_trsm64<T, 64, 4, 2>(k, kb, n, A, lda, info, panel_end, kmax, stream);
+                else
+                    launch_trsm64<T, 16, 8, 1>(k, kb, n, A, lda, info, panel_end, kmax, stream);
+            } else {
+                size_t sm_t = trsm_smem_bytes<T>(kb);
+                const int nbv = (int)cdiv(rest, kTrsmVec);
+                trsm_panel_kernel<T><<<(unsigned)(2 * nbv), kTrsmThreads, sm_t, stream>>>(k, kb, n, A, lda, nbv, info);
+            }
             RBT_LAUNCH_CHECK();
         }
         if (trailing_simt) {
@@ -580,11 +930,11 @@ rbt_status genp_panel_steps(int64_t n, T *A, int64_t lda, int64_t *info, int nb,
 }
 
 template rbt_status genp_panel_steps<double>(int64_t, double *, int64_t, int64_t *, int, int64_t, int64_t, bool,
-                                             cudaStream_t);
+                                             cudaStream_t, int64_t, int *);
 template rbt_status genp_panel_steps<float>(int64_t, float *, int64_t, int64_t *, int, int64_t, int64_t, bool,
-                                            cudaStream_t);
+                                            cudaStream_t, int64_t, int *);
 template rbt_status genp_panel_steps<df64>(int64_t, df64 *, int64_t, int64_t *, int, int64_t, int64_t, bool,
-                                           cudaStream_t);
+                                           cudaStream_t, int64_t, int *);
 
 template <typename T> static rbt_status configure_smem(int nb)
 {

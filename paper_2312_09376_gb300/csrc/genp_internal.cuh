@@ -16,10 +16,14 @@ rbt_status gemm_sub_simt(int64_t M, int64_t N, int K, const T *Am, int64_t lda_a
                          T *C, int64_t ldc, const int64_t *info, cudaStream_t stream);
 
 // Block steps k0, k0+nb, ... < k_end: diagonal factor + both TRSMs, and the
-// trailing update too when trailing_simt is set.
+// trailing update too when trailing_simt is set.  kmax (steps of at most 64
+// columns): receives the exponents that balance the sliced updates, four
+// arrays of kKmax ints (rows before panel_end, rows from it on, columns before
+// it, columns from it on), entry 0 of each for column k0.
+constexpr int kKmax = 512;
 template <typename T>
 rbt_status genp_panel_steps(int64_t n, T *A, int64_t lda, int64_t *info, int nb, int64_t k0, int64_t k_end,
-                            bool trailing_simt, cudaStream_t stream);
+                            bool trailing_simt, cudaStream_t stream, int64_t panel_end = 0, int *kmax = nullptr);
 
 rbt_status genp_configure(int prec, int nb);
 
