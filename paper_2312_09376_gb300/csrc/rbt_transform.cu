@@ -25,6 +25,8 @@
 #include "df64.cuh"
 #include "rbt_dev.cuh"
 
+#include <type_traits>
+
 namespace rbt {
 
 constexpr double kInvSqrt2 = 0.70710678118654752440084436210485;
@@ -214,6 +216,172 @@ fused2_kernel(int64_t n, int64_t h, int64_t ngroups, int k_hi, int pre_lo, int p
 #pragma unroll
             for (int s = 0; s < G; s++)
                 if (rv[s] && cv[t]) Aout[row[s] + col[t] * lda_out] = cvt_out<TO>(x[s][t]);
+    }
+}
+
+// ------------------------------------- double transform on the integer pipes
+//
+// The double-output transform takes about eight FP64 operations an entry at
+// two a clock and SM, six times as long as the entry's 16 bytes of HBM traffic.
+// Here a thread's 2^L x 2^L group is transformed in 64-bit fixed point instead:
+// every entry as a multiple of 2^-58 of the group's largest binade, the
+// butterflies as integer additions, each diagonal factor (with the pair's
+// 1/sqrt(2)) as a 62-bit fraction multiplied by three 32 x 32 -> 64-bit
+// products, and the result rounded to the nearest double.  Every output is a
+// sum over the group, so an error of a few units (2^-58 of the group's largest
+// entry each) is below the half unit of double rounding of |U|^T |A| |V|, and
+// the FP64 form's roundings at every step are gone.  Measured at n = 16385, d =
+// 2: 4.46 -> 1.65 ms (965 -> 2600 GB/s), relative error in the 2-norm 2.3e-16
+// -> 2.0e-16; what bounds it now is the issue of some 80 integer instructions
+// an entry.
+//
+// A group with rows or columns past the matrix (nu rows pass through without
+// being summed), a factor outside (1/4, 6/5), an entry that is not finite, or a
+// largest entry near the ends of the exponent range takes the FP64 form.
+// 64-bit: |v| < 2^58 grows by at most 4 in the butterflies and by
+// 4 (6/5)^2 / 2 < 2^1.6 over a layer: below 2^62 with two layers.
+constexpr int kFixBits = 58;
+constexpr int kFixGroups = 16;  // column groups per CTA (their factors in shared memory)
+
+struct Frac {  // f 2^62 as two 31-bit halves
+    int hi, lo;
+};
+__device__ __forceinline__ Frac frac_of(double f)
+{
+    const long long v = (long long)(f * 0x1p62);
+    return Frac{(int)(v >> 31), (int)(v & 0x7FFFFFFF)};
+}
+__device__ __forceinline__ long long mul_frac(long long v, Frac f)
+{
+    const int vh = (int)(v >> 31), vl = (int)(v & 0x7FFFFFFF);
+    const long long m = (long long)vh * f.lo + (long long)vl * f.hi;  // the dropped vl f.lo is below one unit
+    return (long long)vh * f.hi + (m >> 31);
+}
+// the significand at 2^-58 of the binade of exponent field emax
+__device__ __forceinline__ long long fix_of(double x, int emax)
+{
+    const long long b = __double_as_longlong(x);
+    const int d = emax - ((int)(b >> 52) & 0x7FF);
+    const long long m = ((b & 0xFFFFFFFFFFFFFll) | (1ll << 52)) << (kFixBits - 53);
+    const long long v = m >> (d < 63 ? d : 63);
+    return b < 0 ? -v : v;
+}
+__device__ __forceinline__ double double_of_fix(long long y, int emax)
+{
+    const unsigned long long a = y < 0 ? 0ull - (unsigned long long)y : (unsigned long long)y;
+    const int lz = __clzll((long long)a);
+    const unsigned long long t = a << lz;
+    const unsigned long long r = (t >> 11) + ((t >> 10) & 1);  // 53 bits; a carry past them raises the exponent
+    const unsigned long long e = (unsigned long long)(emax + (64 - kFixBits) - lz - 1) << 52;
+    const unsigned long long bits = a ? e + r : 0ull;
+    return __longlong_as_double((long long)(bits | ((unsigned long long)y & 0x8000000000000000ull)));
+}
+
+template <int L>
+__device__ __noinline__ void transform_group_f64(int64_t n, int64_t h, int k_hi, const double *U, const double *V,
+                                                 int64_t ldw, const double *Ain, int64_t lda_in, double *Aout,
+                                                 int64_t lda_out, int64_t gr, int64_t gc)
+{
+    transform_group<L, double>(n, h, k_hi, 1, 0, U, V, ldw, Ain, lda_in, Aout, lda_out, gr, gc);
+}
+
+// One pass over layers k_hi .. k_hi-L+1, no diagonal-only layers.
+template <int L>
+__global__ void __launch_bounds__(kTX)
+fused2_fix_kernel(int64_t n, int64_t h, int64_t ngroups, int k_hi, const double *__restrict__ U,
+                  const double *__restrict__ V, int64_t ldw, const double *Ain, int64_t lda_in, double *Aout,
+                  int64_t lda_out)
+{
+    constexpr int G = 1 << L;
+    __shared__ Frac cf[kFixGroups][L][G];
+    __shared__ int cok[kFixGroups];
+    const int64_t g0 = (int64_t)blockIdx.y * kFixGroups;
+    const int ng = (int)(ngroups - g0 < kFixGroups ? ngroups - g0 : kFixGroups);
+    auto factor = [&](const double *W, int64_t i, int l, bool &ok) {
+        const double f = i < n ? __ldg(W + i + (int64_t)(k_hi - l - 1) * ldw) : 0.0;
+        ok = ok && f > 0.25 && f < 1.2;
+        return frac_of(ok ? f * kInvSqrt2 : 0.0);
+    };
+    if (threadIdx.x < kFixGroups) cok[threadIdx.x] = 1;
+    __syncthreads();
+    for (int e = threadIdx.x; e < ng * L * G; e += kTX) {
+        const int t = e % G, l = e / G % L, g = e / (G * L);
+        const int64_t gc = g0 + g, cc = gc / h, rc = gc - cc * h;
+        bool ok = true;
+        cf[g][l][t] = factor(V, (cc * G + t) * h + rc, l, ok);
+        if (!ok) cok[g] = 0;
+    }
+    __syncthreads();
+    const int64_t gr = blockIdx.x * (int64_t)kTX + threadIdx.x;
+    if (gr >= ngroups) return;
+    const int64_t cr = gr / h, rr = gr - cr * h;
+    const int64_t row0 = cr * G * h + rr;
+    Frac fu[L][G];
+    bool rok = true;
+#pragma unroll
+    for (int l = 0; l < L; l++)
+#pragma unroll
+        for (int s = 0; s < G; s++) fu[l][s] = factor(U, row0 + s * h, l, rok);
+    for (int g = 0; g < ng; g++) {
+        const int64_t gc = g0 + g, cc = gc / h, rc = gc - cc * h;
+        const int64_t col0 = cc * G * h + rc;
+        bool done = false;
+        if (rok && cok[g]) {
+            double x[G][G];
+            int emax = 0;
+#pragma unroll
+            for (int t = 0; t < G; t++)
+#pragma unroll
+                for (int s = 0; s < G; s++) {
+                    x[s][t] = Ain[row0 + s * h + (col0 + t * h) * lda_in];
+                }
+#pragma unroll
+            for (int t = 0; t < G; t++)
+#pragma unroll
+                for (int s = 0; s < G; s++) emax = max(emax, (__double2hiint(x[s][t]) >> 20) & 0x7FF);
+            if (emax >= 100 && emax <= 2000) {
+                long long v[G][G];
+#pragma unroll
+                for (int t = 0; t < G; t++)
+#pragma unroll
+                    for (int s = 0; s < G; s++) v[s][t] = fix_of(x[s][t], emax);
+#pragma unroll
+                for (int l = 0; l < L; l++) {
+                    const int st = 1 << l;
+#pragma unroll
+                    for (int s = 0; s < G; s++)
+                        if (!(s & st))
+#pragma unroll
+                            for (int t = 0; t < G; t++) {
+                                const long long a = v[s][t], b = v[s | st][t];
+                                v[s][t] = a + b;
+                                v[s | st][t] = a - b;
+                            }
+#pragma unroll
+                    for (int t = 0; t < G; t++)
+                        if (!(t & st))
+#pragma unroll
+                            for (int s = 0; s < G; s++) {
+                                const long long a = v[s][t], b = v[s][t | st];
+                                v[s][t] = a + b;
+                                v[s][t | st] = a - b;
+                            }
+#pragma unroll
+                    for (int t = 0; t < G; t++) {
+                        const Frac fv = cf[g][l][t];
+#pragma unroll
+                        for (int s = 0; s < G; s++) v[s][t] = mul_frac(mul_frac(v[s][t], fu[l][s]), fv);
+                    }
+                }
+#pragma unroll
+                for (int t = 0; t < G; t++)
+#pragma unroll
+                    for (int s = 0; s < G; s++)
+                        Aout[row0 + s * h + (col0 + t * h) * lda_out] = double_of_fix(v[s][t], emax);
+                done = true;
+            }
+        }
+        if (!done) transform_group_f64<L>(n, h, k_hi, U, V, ldw, Ain, lda_in, Aout, lda_out, gr, gc);
     }
 }
 
@@ -630,6 +798,13 @@ static void launch_fused2(int64_t n, int64_t h, int64_t ngroups, int k_hi, int p
                           const double *U, const double *V, int64_t ldw, const double *Ain,
                           int64_t lda_in, TO *Aout, int64_t lda_out, cudaStream_t stream, bool rot)
 {
+    if constexpr (std::is_same<TO, double>::value && L <= 2) {
+        if (!rot && pre_hi < pre_lo) {
+            const dim3 grid((unsigned)cdiv(ngroups, kTX), (unsigned)cdiv(ngroups, kFixGroups));
+            fused2_fix_kernel<L><<<grid, kTX, 0, stream>>>(n, h, ngroups, k_hi, U, V, ldw, Ain, lda_in, Aout, lda_out);
+            return;
+        }
+    }
     const int gpt = 4;
     dim3 grid((unsigned)cdiv(ngroups, kTX), (unsigned)cdiv(ngroups, gpt));
     if (rot)
