@@ -61,7 +61,7 @@ typedef enum {
 /* Working precision of the factorization. */
 typedef enum {
     RBT_F64 = 0,   /* double storage and arithmetic; rbt_solve with nb = 0 and
-                      n >= 1024 runs the factorization's updates by exact digit
+                      n >= 768 runs the factorization's updates by exact digit
                       slicing on the BF16 tensor cores (nine 7-bit digits, 63
                       bits relative to each row's and column's largest entry)
                       when A~ is dense enough for that to be no less accurate

@@ -9,6 +9,7 @@
 #include <cmath>
 
 #include "common.cuh"
+#include "gemm_tc.cuh"
 #include "genp_internal.cuh"
 
 namespace rbt {
@@ -221,10 +222,39 @@ rbt_status rbt_solve_adjoint(const rbt_opts *opts, const rbt_info *fwd, int64_t 
         *out = h != 0;
         return RBT_OK;
     };
-    RBT_CUDA_TRY(cudaMemcpy2DAsync(Y, ldy * 8, G, ldg * 8, n * 8, nrhs, cudaMemcpyDeviceToDevice, s));
-    rbt_status st = corr(Y, ldy, false);
+    // many right-hand sides: residuals by sliced products, as in rbt_solve
+    // (the first one's ||A^T|| from one column's pass)
+    void *fac = w + L.fac;
+    const size_t fac_bytes = L.sol - L.fac;
+    bool sliced_res = false;
+    rbt_status st = sliced_residual(n, nrhs, A, lda, fac, fac_bytes, &sliced_res, s);
     if (st != RBT_OK) return st;
-    st = resid_t(n, nrhs, A, lda, Y, ldy, G, ldg, R, n, scal + 2, true, scal + 3, s);
+    int *res_status = (int *)((char *)fac + fac_bytes / 256 * 256 - 256);
+    int h_res = 0;
+    // "no failed pivot" for the update kernel (with another nrhs than the
+    // forward call's, its own word lies elsewhere)
+    if (sliced_res) RBT_CUDA_TRY(cudaMemsetAsync(w + L.info, 0xff, sizeof(int64_t), s));
+    auto residual = [&](bool want_norm) -> rbt_status {
+        if (!sliced_res) return resid_t(n, nrhs, A, lda, Y, ldy, G, ldg, R, n, scal + 2, want_norm, scal + 3, s);
+        if (want_norm) {
+            rbt_status e = resid_t(n, 1, A, lda, Y, ldy, G, ldg, R, n, scal + 2, true, scal + 3, s);
+            if (e != RBT_OK) return e;
+        }
+        ProfScope ps(kProfResidual, s);
+        RBT_CUDA_TRY(cudaMemsetAsync(res_status, 0, sizeof(int), s));
+        RBT_CUDA_TRY(cudaMemcpy2DAsync(R, n * 8, G, ldg * 8, n * 8, nrhs, cudaMemcpyDeviceToDevice, s));
+        rbt_status e = oz_residual(n, nrhs, A, lda, true, Y, ldy, R, n, (const int64_t *)(w + L.info), fac, res_status, s);
+        if (e != RBT_OK) return e;
+        RBT_CUDA_TRY(cudaMemcpyAsync(&h_res, res_status, sizeof(int), cudaMemcpyDeviceToHost, s));
+        RBT_CUDA_TRY(cudaMemsetAsync(scal + 3, 0, 8, s));
+        berr_t_kernel<<<(unsigned)nrhs, 256, 0, s>>>(n, R, n, Y, ldy, G, ldg, scal + 2, scal + 3);
+        RBT_LAUNCH_CHECK();
+        return RBT_OK;
+    };
+    RBT_CUDA_TRY(cudaMemcpy2DAsync(Y, ldy * 8, G, ldg * 8, n * 8, nrhs, cudaMemcpyDeviceToDevice, s));
+    st = corr(Y, ldy, false);
+    if (st != RBT_OK) return st;
+    st = residual(true);
     if (st != RBT_OK) return st;
     double berr = 0.0;
     RBT_CUDA_TRY(cudaMemcpyAsync(&berr, scal + 3, 8, cudaMemcpyDeviceToHost, s));
@@ -236,7 +266,7 @@ rbt_status rbt_solve_adjoint(const rbt_opts *opts, const rbt_info *fwd, int64_t 
         if (st != RBT_OK) return st;
         st = add_block(n, nrhs, R, n, Y, ldy, s);
         if (st != RBT_OK) return st;
-        st = resid_t(n, nrhs, A, lda, Y, ldy, G, ldg, R, n, scal + 2, false, scal + 3, s);
+        st = residual(false);
         if (st != RBT_OK) return st;
         double prev = berr;
         RBT_CUDA_TRY(cudaMemcpyAsync(&berr, scal + 3, 8, cudaMemcpyDeviceToHost, s));
@@ -247,7 +277,7 @@ rbt_status rbt_solve_adjoint(const rbt_opts *opts, const rbt_info *fwd, int64_t 
     bool to = false;
     st = timed_out(&to);
     if (st != RBT_OK) return st;
-    if (to) return RBT_ERR_TIMEOUT;
+    if (to || h_res) return RBT_ERR_TIMEOUT;
     info->iters = it;
     info->berr = berr;
     info->status = berr <= opts->tol ? RBT_OK : RBT_NOT_CONVERGED;

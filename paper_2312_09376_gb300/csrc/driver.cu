@@ -83,8 +83,8 @@ void prof_record(int cls, cudaStream_t s, bool begin)
 }
 
 // From this order a double factorization runs its updates on the tensor cores:
-// per solve, SIMT / sliced, n = 1003: 4.20 / 4.28 ms; 4001: 48.2 / 17.7 ms.
-constexpr int64_t kSliced64Min = 1024;
+// per solve, FP64 pipe / sliced, n = 1003: 3.71 / 2.9 ms; 4001: 48.2 / 13.5 ms.
+constexpr int64_t kSliced64Min = 768;
 
 static int default_nb(int prec)
 {
@@ -230,6 +230,27 @@ rbt_status factor_copy(int64_t n, int prec, void *At, int64_t ldt, int64_t *d_in
     RBT_CUDA_TRY(cudaMemsetAsync(d_info, 0xff, sizeof(int64_t), s));  // -1
     return genp_factor_impl(n, prec, At, ldt, d_info, fac, fac_bytes, nb, s, even);
 }
+
+}  // namespace
+
+namespace rbt {
+
+// Fewest right-hand sides for sliced residuals: at n = 8197 the FP64 pipe takes
+// 0.14 ms a right-hand side (4.5 ms for 32), the sliced form 2.1 ms for up to 48.
+constexpr int64_t kSlicedResRhs = 16;
+
+rbt_status sliced_residual(int64_t n, int64_t nrhs, const double *A, int64_t lda, void *scratch, size_t bytes, bool *yes,
+                           cudaStream_t stream)
+{
+    *yes = false;
+    if (n < kSliced64Min || nrhs < kSlicedResRhs || n > INT32_MAX / 9 || nrhs > INT32_MAX / 9) return RBT_OK;
+    if (bytes < std::max(oz_residual_workspace(n, nrhs), spread_workspace(n))) return RBT_OK;
+    return evenly_spread(n, A, lda, scratch, yes, stream);
+}
+
+}  // namespace rbt
+
+namespace {
 
 // dX = V A~^{-1} U^T R, in place in R
 rbt_status correction(int64_t n, int64_t nrhs, int d, int64_t align, int kind, const double *U, const double *V, int prec,
@@ -442,6 +463,26 @@ rbt_status rbt_solve(const rbt_opts *opts, int64_t n, int64_t nrhs, const double
     // here and read after every step: a timeout anywhere in this call sticks
     RBT_CUDA_TRY(cudaMemsetAsync(sol, 0, sizeof(int), s));
 
+    // many right-hand sides: residuals by sliced products, in the scratch of
+    // the factorization (its last 256 bytes: their status word)
+    bool sliced_res = false;
+    st = sliced_residual(n, nrhs, A, lda, fac, fac_bytes, &sliced_res, s);
+    if (st != RBT_OK) return st;
+    int *res_status = (int *)((char *)fac + fac_bytes / 256 * 256 - 256);
+    int h_res = 0;
+    auto residual = [&]() -> rbt_status {
+        if (!sliced_res) return residual_impl(n, nrhs, A, lda, X, ldx, B, ldb, R, n, scal, scal + 1, res, s);
+        {
+            ProfScope ps(kProfResidual, s);
+            RBT_CUDA_TRY(cudaMemsetAsync(res_status, 0, sizeof(int), s));
+            RBT_CUDA_TRY(cudaMemcpy2DAsync(R, n * 8, B, ldb * 8, n * 8, nrhs, cudaMemcpyDeviceToDevice, s));
+            rbt_status e = oz_residual(n, nrhs, A, lda, false, X, ldx, R, n, d_info, fac, res_status, s);
+            if (e != RBT_OK) return e;
+        }
+        RBT_CUDA_TRY(cudaMemcpyAsync(&h_res, res_status, sizeof(int), cudaMemcpyDeviceToHost, s));
+        return backward_error(n, nrhs, X, ldx, B, ldb, R, n, scal, scal + 1, s);
+    };
+
     // 1. butterflies and the transformed working matrix (Eq. precond step 1)
     st = opts->kind == RBT_KIND_ROTATION ? rbt_generate_rot(n, d, align, opts->seed, U, V, n, s)
                                          : rbt_generate(n, d, opts->seed, U, V, n, s);
@@ -459,7 +500,7 @@ rbt_status rbt_solve(const rbt_opts *opts, int64_t n, int64_t nrhs, const double
     RBT_CUDA_TRY(cudaMemcpy2DAsync(X, ldx * 8, B, ldb * 8, n * 8, nrhs, cudaMemcpyDeviceToDevice, s));
     st = correction(n, nrhs, d, align, opts->kind, U, V, prec, At, ldt, X, ldx, sol, false, s);
     if (st != RBT_OK) return st;
-    st = residual_impl(n, nrhs, A, lda, X, ldx, B, ldb, R, n, scal, scal + 1, res, s);
+    st = residual();
     if (st != RBT_OK) return st;
     int64_t h_info = -1;
     double berr = 0.0;
@@ -468,7 +509,7 @@ rbt_status rbt_solve(const rbt_opts *opts, int64_t n, int64_t nrhs, const double
     RBT_CUDA_TRY(cudaMemcpyAsync(&berr, scal + 1, 8, cudaMemcpyDeviceToHost, s));
     RBT_CUDA_TRY(cudaMemcpyAsync(&h_wait, sol, 4, cudaMemcpyDeviceToHost, s));
     RBT_CUDA_TRY(cudaStreamSynchronize(s));
-    if (h_wait) return RBT_ERR_TIMEOUT;
+    if (h_wait || h_res) return RBT_ERR_TIMEOUT;
     if (h_info == -2) return RBT_ERR_TIMEOUT;
 
     int cur_prec = prec;
@@ -537,10 +578,11 @@ rbt_status rbt_solve(const rbt_opts *opts, int64_t n, int64_t nrhs, const double
             RBT_CUDA_TRY(cudaMemcpy2DAsync(X, ldx * 8, B, ldb * 8, n * 8, nrhs, cudaMemcpyDeviceToDevice, s));
             st = correction(n, nrhs, d, align, opts->kind, U, V, cur_prec, cur_At, cur_ldt, X, ldx, sol, false, s);
             if (st != RBT_OK) return st;
-            st = residual_impl(n, nrhs, A, lda, X, ldx, B, ldb, R, n, scal, scal + 1, res, s);
+            st = residual();
             if (st != RBT_OK) return st;
             RBT_CUDA_TRY(cudaMemcpyAsync(&berr, scal + 1, 8, cudaMemcpyDeviceToHost, s));
             RBT_CUDA_TRY(cudaStreamSynchronize(s));
+            if (h_res) return RBT_ERR_TIMEOUT;
             continue;
         }
         if (opts->refine_mode == RBT_REFINE_GMRES) {
@@ -559,13 +601,13 @@ rbt_status rbt_solve(const rbt_opts *opts, int64_t n, int64_t nrhs, const double
             st = add_block(n, nrhs, R, n, X, ldx, s);
             if (st != RBT_OK) return st;
         }
-        st = residual_impl(n, nrhs, A, lda, X, ldx, B, ldb, R, n, scal, scal + 1, res, s);
+        st = residual();
         if (st != RBT_OK) return st;
         prev = berr;
         RBT_CUDA_TRY(cudaMemcpyAsync(&berr, scal + 1, 8, cudaMemcpyDeviceToHost, s));
         RBT_CUDA_TRY(cudaMemcpyAsync(&h_wait, sol, 4, cudaMemcpyDeviceToHost, s));
         RBT_CUDA_TRY(cudaStreamSynchronize(s));
-        if (h_wait) return RBT_ERR_TIMEOUT;
+        if (h_wait || h_res) return RBT_ERR_TIMEOUT;
         iters++;
         attempt_iters++;
     }

@@ -29,7 +29,7 @@
 // same binade (on RBT-transformed GENP panels the bound relative to the
 // entrywise one drops from about 2^12 to 2^4 in the median).
 //
-// Double operands (RBT_F64, from n = 1024) take the same route with nine
+// Double operands (RBT_F64, from n = 768) take the same route with nine
 // digits: 63 bits relative to the row and column maxima, ten more than an
 // entry has, 45 products, K <= 448 (9 K 2^12 <= 2^24), 48-column tiles (nine
 // accumulators in TMEM), the fold in 64-bit integers.  Measured against the
@@ -720,6 +720,7 @@ template <int S> struct Operands {
     const elem_t<S> *A, *B;
     elem_t<S> *C;
     const int *ka, *ka2, *kb;
+    bool ta = false;  // A is stored as its transpose (K x M)
 };
 
 // One or two products of the same K and leading dimensions: the digit slices
@@ -736,11 +737,11 @@ static rbt_status products(int count, const Operands<S> *op, const Slices *sl, i
         const int per = K <= 64 ? 16 : 8;  // columns of B per CTA
         int64_t blocks = 0;
         for (int i = 0; i < count; i++) {
-            const int nra = (int)(sl[i].Mp / kSliceRows), nrb = (int)cdiv(sl[i].Np, per);
+            const int nra = (int)(op[i].ta ? cdiv(sl[i].Mp, per) : sl[i].Mp / kSliceRows), nrb = (int)cdiv(sl[i].Np, per);
             jobs.job[2 * i] = {op[i].A, lda, (int)op[i].M, (int)sl[i].Mp, op[i].ka, op[i].ka2, op[i].kb,
-                               sl[i].sa, sl[i].ea, 1, nra};
+                               sl[i].sa, sl[i].ea, op[i].ta ? 0 : 1, 1, nra};
             jobs.job[2 * i + 1] = {op[i].B, ldb, (int)op[i].N, (int)sl[i].Np, op[i].ka, op[i].ka2, op[i].kb,
-                                   sl[i].sb, sl[i].fb, 0, nrb};
+                                   sl[i].sb, sl[i].fb, 0, -1, nrb};
             blocks += nra + nrb;
         }
         jobs.K = (int)K;
@@ -778,7 +779,7 @@ static rbt_status products(int count, const Operands<S> *op, const Slices *sl, i
 template <int S>
 static rbt_status update(int64_t M, int64_t N, int64_t K, const elem_t<S> *A, int64_t lda, const elem_t<S> *B,
                          int64_t ldb, elem_t<S> *C, int64_t ldc, const int64_t *info, void *work, void *status,
-                         unsigned max_ctas, cudaStream_t stream)
+                         unsigned max_ctas, cudaStream_t stream, bool ta = false)
 {
     rbt_status s = configure<S>();
     if (s != RBT_OK) return s;
@@ -787,12 +788,12 @@ static rbt_status update(int64_t M, int64_t N, int64_t K, const elem_t<S> *A, in
         ProfScope pslice(kProfSlice, stream);
         // both exponent arrays start at kNoExp (every byte 0x80)
         RBT_CUDA_TRY(cudaMemsetAsync(sl.ka, 0x80, (size_t)rup(sl.Kp * 4, 256) * 2, stream));
-        const int ca = (int)cdiv(M, 4096), na = ca * (int)K;
-        kexp_kernel<elem_t<S>><<<(unsigned)(na + cdiv(N, 64)), 256, 0, stream>>>((int)M, (int)K, (int)N, ca, na, A, lda,
-                                                                              B, ldb, sl.ka, sl.kb);
+        const int ca = (int)cdiv(M, 4096), na = ta ? (int)cdiv(M, 64) : ca * (int)K;
+        kexp_kernel<elem_t<S>><<<(unsigned)(na + cdiv(N, 64)), 256, 0, stream>>>((int)M, (int)K, (int)N, ca, na, ta, A,
+                                                                              lda, B, ldb, sl.ka, sl.kb);
         RBT_LAUNCH_CHECK();
     }
-    const Operands<S> op = {M, N, A, B, C, sl.ka, sl.ka, sl.kb};
+    const Operands<S> op = {M, N, A, B, C, sl.ka, sl.ka, sl.kb, ta};
     return products<S, false>(1, &op, &sl, K, lda, ldb, ldc, info, status, max_ctas, stream);
 }
 
@@ -812,6 +813,29 @@ rbt_status oz_update(int64_t M, int64_t N, int64_t K, const df64 *A, int64_t lda
     const unsigned ctas = max_ctas ? max_ctas : (unsigned)device_sm_count();
     return digits == 7 ? update<7>(M, N, K, A, lda, B, ldb, C, ldc, info, work, status, ctas, stream)
                        : update<8>(M, N, K, A, lda, B, ldb, C, ldc, info, work, status, ctas, stream);
+}
+
+size_t oz_residual_workspace(int64_t n, int64_t nrhs)
+{
+    return oz_update_workspace(n, nrhs, oz::KMAX<9>, oz::kDigits64) + 256;
+}
+
+// R (n x nrhs) -= A X, or A^T X, in double by nine-digit sliced products over
+// pieces of 448 of the inner dimension: each reads A once, whatever the number
+// of right-hand sides, where the FP64 pipe takes n^2 nrhs multiply-adds at two
+// a clock and SM (3.4 ms for 32 at n = 8197).  *status (device, cleared by the
+// caller) becomes nonzero when a device wait gave up.
+rbt_status oz_residual(int64_t n, int64_t nrhs, const double *A, int64_t lda, bool trans, const double *X, int64_t ldx,
+                       double *R, int64_t ldr, const int64_t *info, void *work, int *status, cudaStream_t stream)
+{
+    using namespace oz;
+    for (int64_t k = 0; k < n; k += KMAX<9>) {
+        const int64_t K = std::min<int64_t>(n - k, KMAX<9>);
+        const rbt_status s = update<9>(n, nrhs, K, trans ? A + k : A + k * lda, lda, X + k, ldx, R, ldr, info, work, status,
+                                       (unsigned)device_sm_count(), stream, trans);
+        if (s != RBT_OK) return s;
+    }
+    return RBT_OK;
 }
 
 rbt_status oz_status_to_info(void *status, int64_t *info, cudaStream_t stream)

@@ -24,6 +24,9 @@ rbt_status oz_update(int64_t M, int64_t N, int64_t K, const df64 *A, int64_t lda
                      cudaStream_t stream, unsigned max_ctas = 0);
 rbt_status oz_status_to_info(void *status, int64_t *info, cudaStream_t stream);
 size_t oz_factor_workspace(int64_t n);
+size_t oz_residual_workspace(int64_t n, int64_t nrhs);
+rbt_status oz_residual(int64_t n, int64_t nrhs, const double *A, int64_t lda, bool trans, const double *X, int64_t ldx,
+                       double *R, int64_t ldr, const int64_t *info, void *work, int *status, cudaStream_t stream);
 rbt_status genp_factor_oz64(int64_t n, double *A, int64_t lda, int64_t *info, void *work, size_t work_bytes,
                             cudaStream_t stream);
 rbt_status genp_factor_oz(int64_t n, df64 *A, int64_t lda, int64_t *info, void *work, size_t work_bytes, int digits,

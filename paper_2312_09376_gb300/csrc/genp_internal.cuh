@@ -36,6 +36,14 @@ rbt_status norm_inf_impl(int64_t n, const double *A, int64_t lda, double *d_out,
 rbt_status residual_impl(int64_t n, int64_t nrhs, const double *A, int64_t lda, const double *X, int64_t ldx,
                          const double *B, int64_t ldb, double *R, int64_t ldr, const double *d_anorm,
                          double *d_berr, double *part, cudaStream_t stream);
+// d_berr <- the largest backward error over the columns, from R = B - A X
+rbt_status backward_error(int64_t n, int64_t nrhs, const double *X, int64_t ldx, const double *B, int64_t ldb,
+                          const double *R, int64_t ldr, const double *d_anorm, double *d_berr, cudaStream_t stream);
+// Whether a solve's residuals go through oz_residual (scratch: its bytes, free
+// between factorizations): many right-hand sides, and A's rows and columns
+// filled with entries of like size (spread.cu; synchronizes).
+rbt_status sliced_residual(int64_t n, int64_t nrhs, const double *A, int64_t lda, void *scratch, size_t bytes, bool *yes,
+                           cudaStream_t stream);
 rbt_status add_block(int64_t n, int64_t nrhs, const double *D, int64_t ldd, double *X, int64_t ldx,
                      cudaStream_t stream);
 

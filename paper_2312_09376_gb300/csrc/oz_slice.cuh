@@ -172,27 +172,34 @@ __device__ __forceinline__ __nv_bfloat16 bf16_of_digit(int r) { return __int2bfl
 // ka[k] = max over rows of E(A_ik), kb[k] = max over columns of E(B_kj).  (A
 // factorization gets them from its panel TRSMs instead.)  One launch for both:
 // blocks [0, na) take A (block b: column k = b / ca, rows of chunk b % ca,
-// 4096 rows each), the rest take B (64 columns each; threads over k).
+// 4096 rows each; with ta 64 of its rows, stored as columns), the rest take B
+// (64 columns each; threads over k).
 template <typename TE>
-__global__ void __launch_bounds__(256) kexp_kernel(int M, int K, int N, int ca, int na, const TE *__restrict__ A,
-                                                   int64_t lda, const TE *__restrict__ B, int64_t ldb, int *ka,
-                                                   int *kb)
+__global__ void __launch_bounds__(256) kexp_kernel(int M, int K, int N, int ca, int na, int ta,
+                                                   const TE *__restrict__ A, int64_t lda, const TE *__restrict__ B,
+                                                   int64_t ldb, int *ka, int *kb)
 {
     const int b = blockIdx.x;
-    if (b < na) {
+    if (b < na && !ta) {
         const int k = b / ca, chunk = b % ca;
         int e = kNoExp;
         const int r1 = min(M, (chunk + 1) * 4096);
+#pragma unroll 8
         for (int r = chunk * 4096 + threadIdx.x; r < r1; r += 256) e = max(e, finite_exp(exp_of(A[r + (int64_t)k * lda])));
         for (int o = 16; o > 0; o >>= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
         if (threadIdx.x % 32 == 0 && e > kNoExp) atomicMax(ka + k, e);
         return;
     }
-    const int c0 = (b - na) * 64, c1 = min(N, c0 + 64);
+    // B, or an A given as its transpose (ta: K x M): 64 columns
+    const bool is_a = b < na;
+    const TE *src = is_a ? A : B;
+    const int64_t ld = is_a ? lda : ldb;
+    const int c0 = (is_a ? b : b - na) * 64, c1 = min(is_a ? M : N, c0 + 64);
     for (int k = threadIdx.x; k < K; k += 256) {
         int e = kNoExp;
-        for (int c = c0; c < c1; c++) e = max(e, finite_exp(exp_of(B[k + (int64_t)c * ldb])));
-        if (e > kNoExp) atomicMax(kb + k, e);
+#pragma unroll 8
+        for (int c = c0; c < c1; c++) e = max(e, finite_exp(exp_of(src[k + (int64_t)c * ld])));
+        if (e > kNoExp) atomicMax((is_a ? ka : kb) + k, e);
     }
 }
 
@@ -207,8 +214,9 @@ __device__ __forceinline__ int kshift(int a, int b)
 
 // ---- slicing
 
-// One operand: A (rows x K, column-major; the slices' rows are its rows) or B
-// (K x rows, column-major; its columns).  Slice p goes to rows p rows_p ..
+// One operand: stored rows x K (by_rows; the slices' rows are its rows) or K x
+// rows (its columns), column-major.  Its k are scaled by 2^(sign t_k), sign 1
+// for A (or its transpose stored K x M) and -1 for B.  Slice p goes to rows p rows_p ..
 // of a K-major [S rows_p][Kp] bf16 array (zeros past rows and K), the row
 // exponents to exps.  The balancing exponents of A's columns are the larger
 // of ka and ka2, those of B's rows kb.
@@ -219,7 +227,7 @@ template <typename TE> struct SliceJob {
     const int *ka, *ka2, *kb;
     __nv_bfloat16 *out;
     int *exps;
-    int is_a, blocks;
+    int by_rows, sign, blocks;
 };
 template <typename TE> struct SliceJobs {
     SliceJob<TE> job[4];
@@ -272,7 +280,7 @@ __global__ void __launch_bounds__(256) slice_kernel(const __grid_constant__ Slic
     auto shifts = [&]() {  // t_k of every k
         for (int k = tid; k < Kp; k += 256) ts[k] = k < K ? kshift(max(J.ka[k], J.ka2[k]), J.kb[k]) : 0;
     };
-    if (J.is_a) {
+    if (J.by_rows) {
         const int ld_t = Kp + 2, r = tid % kSliceRows, kl = tid / kSliceRows;
         const int m = blk * kSliceRows + r;
 #pragma unroll 8
@@ -316,6 +324,7 @@ __global__ void __launch_bounds__(256) slice_kernel(const __grid_constant__ Slic
             }
         shifts();
         __syncthreads();
+        const int sg = J.sign;
         int emax = kNoExp;  // max over k of E(B_kc 2^-t_k)
 #pragma unroll
         for (int i = 0; i < NI; i++)
@@ -323,7 +332,7 @@ __global__ void __launch_bounds__(256) slice_kernel(const __grid_constant__ Slic
             for (int u = 0; u < 4; u++) {
                 const int k = 4 * l + 4 * LPC * i + u;
                 const int e = exp_of(v[i][u]);
-                if (k < K && e != kNoExp) emax = max(emax, e == kBadExp ? e : e - ts[k]);
+                if (k < K && e != kNoExp) emax = max(emax, e == kBadExp ? e : e + sg * ts[k]);
             }
 #pragma unroll
         for (int o = LPC / 2; o > 0; o >>= 1) emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, o));
@@ -336,7 +345,7 @@ __global__ void __launch_bounds__(256) slice_kernel(const __grid_constant__ Slic
             if (k >= Kp) break;
             Fields<S> f[4];
 #pragma unroll
-            for (int u = 0; u < 4; u++) f[u] = e != kBadExp ? fields<S, WIDE>(v[i][u], e + ts[k + u]) : no_digits<S, WIDE>();
+            for (int u = 0; u < 4; u++) f[u] = e != kBadExp ? fields<S, WIDE>(v[i][u], e - sg * ts[k + u]) : no_digits<S, WIDE>();
             store4<S, WIDE>(f, J.out + (int64_t)c * Kp + k, slice);
         }
     }

@@ -176,6 +176,15 @@ rbt_status norm_inf_impl(int64_t n, const double *A, int64_t lda, double *d_out,
     return RBT_OK;
 }
 
+rbt_status backward_error(int64_t n, int64_t nrhs, const double *X, int64_t ldx, const double *B, int64_t ldb,
+                          const double *R, int64_t ldr, const double *d_anorm, double *d_berr, cudaStream_t stream)
+{
+    RBT_CUDA_TRY(cudaMemsetAsync(d_berr, 0, sizeof(double), stream));
+    berr_kernel<<<(unsigned)nrhs, 256, 0, stream>>>(n, R, ldr, X, ldx, B, ldb, d_anorm, d_berr);
+    RBT_LAUNCH_CHECK();
+    return RBT_OK;
+}
+
 rbt_status residual_impl(int64_t n, int64_t nrhs, const double *A, int64_t lda, const double *X, int64_t ldx,
                          const double *B, int64_t ldb, double *R, int64_t ldr, const double *d_anorm,
                          double *d_berr, double *part, cudaStream_t stream)
@@ -191,12 +200,7 @@ rbt_status residual_impl(int64_t n, int64_t nrhs, const double *A, int64_t lda, 
     RBT_LAUNCH_CHECK();
     residual_reduce_kernel<<<(unsigned)cdiv(n * nrhs, 256), 256, 0, stream>>>(n, nrhs, nch, part, B, ldb, R, ldr);
     RBT_LAUNCH_CHECK();
-    if (d_berr) {
-        RBT_CUDA_TRY(cudaMemsetAsync(d_berr, 0, sizeof(double), stream));
-        berr_kernel<<<(unsigned)nrhs, 256, 0, stream>>>(n, R, ldr, X, ldx, B, ldb, d_anorm, d_berr);
-        RBT_LAUNCH_CHECK();
-    }
-    return RBT_OK;
+    return d_berr ? backward_error(n, nrhs, X, ldx, B, ldb, R, ldr, d_anorm, d_berr, stream) : RBT_OK;
 }
 
 }  // namespace rbt
