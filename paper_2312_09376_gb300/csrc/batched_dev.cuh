@@ -25,6 +25,10 @@ struct SysDesc {
 
 constexpr int kMaxRhsChunk = 8;
 constexpr int kTile = 64;  // trailing-update tile
+constexpr int kTileB = kTile + 4;  // its row of U12 in shared memory: four columns a thread in one read, 16-byte aligned
+// shared memory of a solve, in elements of the widest type: the diagonal
+// block, L21 of a tile, U12 of a tile
+template <int NB> constexpr int kSmemElems = NB * NB + kTile * NB + kTileB * NB;
 // Threads per SM the kernels' launch bounds ask room for: 512, i.e. at most
 // 128 registers a thread, two CTAs of 256 threads (or four of 128) per SM.
 // Uncapped, the compiler gives the whole solver 255 registers (one CTA per
@@ -153,14 +157,23 @@ __device__ int64_t cta_genp(int64_t n, T *A, T *s_diag, T *s_a, T *s_b, int *s_f
                 if (j < kb) A[r + (k0 + j) * n] = x[j];
         }
         __syncthreads();
-        // A22 -= L21 U12, 64 x 64 tiles, each thread a (64*64/NT) register tile
+        // A22 -= L21 U12, 64 x 64 tiles, each thread a (64*64/NT) register
+        // tile: TW rows 64 / TW apart (coalesced) by TH columns.  Down a column
+        // of tiles U12's part stays in shared memory.  In float the columns are
+        // neighbours (one or two shared reads for all) and a tile's block of
+        // A22 is read before its multiply-adds, which hide the latency; in the
+        // wider types the multiply-adds are the bound (double 158.5 ms a batch,
+        // 160.1 with this form; float 84.4 -> 80.7).
+        constexpr bool kPre = sizeof(T) == 4;
         const int64_t rest = n - r0;
         const int64_t nt = (rest + kTile - 1) / kTile;
         constexpr int TPR = kTile * kTile / NT;  // outputs per thread
-        constexpr int TW = (TPR >= 16) ? 4 : 2;  // register tile TW x (TPR / TW)
+        constexpr int TW = 4;                    // register tile TW x (TPR / TW)
         constexpr int TH = TPR / TW;
         constexpr int GX = kTile / TW;           // threads along rows
         const int tx = tid % GX, ty = tid / GX;
+        auto b_at = [](int p, int j) { return kPre ? p * kTileB + j : p + j * NB; };
+        auto col = [&](int b) { return kPre ? ty * TH + b : ty + b * (NT / GX); };
         for (int64_t t = 0; t < nt * nt; t++) {
             const int64_t ti = t % nt, tj = t / nt;
             const int64_t i0 = r0 + ti * kTile, j0 = r0 + tj * kTile;
@@ -168,22 +181,27 @@ __device__ int64_t cta_genp(int64_t n, T *A, T *s_diag, T *s_a, T *s_b, int *s_f
                 int i = e % kTile, p = e / kTile;
                 s_a[i + p * kTile] = (i0 + i < n) ? A[(i0 + i) + (k0 + p) * n] : T(0);
             }
-            for (int e = tid; e < kTile * kb; e += NT) {
-                int p = e % kb, j = e / kb;
-                s_b[p + j * NB] = (j0 + j < n) ? A[(k0 + p) + (j0 + j) * n] : T(0);
-            }
+            if (ti == 0)
+                for (int e = tid; e < kTile * kb; e += NT) {
+                    int p = e % kb, j = e / kb;
+                    s_b[b_at(p, j)] = (j0 + j < n) ? A[(k0 + p) + (j0 + j) * n] : T(0);
+                }
+            T c[kPre ? TW : 1][kPre ? TH : 1], acc[TW][TH];
+#pragma unroll
+            for (int b = 0; b < TH; b++)
+#pragma unroll
+                for (int a = 0; a < TW; a++) {
+                    const int64_t i = i0 + tx + a * GX, j = j0 + col(b);
+                    if constexpr (kPre) c[a][b] = (i < n && j < n) ? A[i + j * n] : T(0);
+                    acc[a][b] = T(0);
+                }
             __syncthreads();
-            T acc[TW][TH];
-#pragma unroll
-            for (int a = 0; a < TW; a++)
-#pragma unroll
-                for (int b = 0; b < TH; b++) acc[a][b] = T(0);
             for (int p = 0; p < kb; p++) {
                 T ra[TW], rb[TH];
 #pragma unroll
                 for (int a = 0; a < TW; a++) ra[a] = s_a[(tx + a * GX) + p * kTile];
 #pragma unroll
-                for (int b = 0; b < TH; b++) rb[b] = s_b[p + (ty + b * (NT / GX)) * NB];
+                for (int b = 0; b < TH; b++) rb[b] = s_b[b_at(p, col(b))];
 #pragma unroll
                 for (int a = 0; a < TW; a++)
 #pragma unroll
@@ -191,12 +209,16 @@ __device__ int64_t cta_genp(int64_t n, T *A, T *s_diag, T *s_a, T *s_b, int *s_f
             }
 #pragma unroll
             for (int b = 0; b < TH; b++) {
-                int64_t j = j0 + ty + b * (NT / GX);
+                const int64_t j = j0 + col(b);
                 if (j >= n) continue;
 #pragma unroll
                 for (int a = 0; a < TW; a++) {
-                    int64_t i = i0 + tx + a * GX;
-                    if (i < n) A[i + j * n] -= acc[a][b];
+                    const int64_t i = i0 + tx + a * GX;
+                    if constexpr (kPre) {
+                        if (i < n) A[i + j * n] = c[a][b] - acc[a][b];
+                    } else {
+                        if (i < n) A[i + j * n] -= acc[a][b];
+                    }
                 }
             }
             __syncthreads();
@@ -243,14 +265,58 @@ __device__ __forceinline__ void cta_load_block(int kb, const T *LU, int64_t n, i
     for (int e = threadIdx.x; e < kb * kb; e += NT) s_blk[e] = LU[(k0 + e % kb) + (k0 + e / kb) * n];
 }
 
+// Rows [lo, hi) of X(:, c0 .. c0 + NC) -= LU(:, k0 .. k0 + kb) times the
+// block's solved rows (in s_x): one row per thread, its entries of LU read
+// once for NC right-hand sides.
+template <typename T, int NT, int NB, int NC>
+__device__ __forceinline__ void rows_minus_block(int64_t n, int64_t lo, int64_t hi, int64_t k0, int kb, int64_t c0,
+                                                 const T *LU, T *X, const T *s_x)
+{
+    for (int64_t r = lo + threadIdx.x; r < hi; r += NT) {
+        T s[NC];
+#pragma unroll
+        for (int c = 0; c < NC; c++) s[c] = T(0);
+#pragma unroll 4
+        for (int p = 0; p < kb; p++) {
+            const T m = LU[r + (k0 + p) * n];
+#pragma unroll
+            for (int c = 0; c < NC; c++) s[c] = fma(m, s_x[c * NB + p], s[c]);
+        }
+#pragma unroll
+        for (int c = 0; c < NC; c++) X[r + (c0 + c) * n] -= s[c];
+    }
+}
+
+// The same for every right-hand side, in chunks of 8, 4, 2 and 1.  s_x: 8 NB
+// elements of shared memory.
+template <typename T, int NT, int NB>
+__device__ __forceinline__ void cta_minus_block(int64_t n, int64_t nrhs, int64_t lo, int64_t hi, int64_t k0, int kb,
+                                                const T *LU, T *X, T *s_x)
+{
+    for (int64_t c0 = 0; c0 < nrhs;) {
+        const int64_t left = nrhs - c0;
+        const int nc = left >= 8 ? 8 : left >= 4 ? 4 : left >= 2 ? 2 : 1;
+        for (int e = threadIdx.x; e < kb * nc; e += NT) s_x[e / kb * NB + e % kb] = X[(k0 + e % kb) + (c0 + e / kb) * n];
+        __syncthreads();
+        switch (nc) {
+        case 8: rows_minus_block<T, NT, NB, 8>(n, lo, hi, k0, kb, c0, LU, X, s_x); break;
+        case 4: rows_minus_block<T, NT, NB, 4>(n, lo, hi, k0, kb, c0, LU, X, s_x); break;
+        case 2: rows_minus_block<T, NT, NB, 2>(n, lo, hi, k0, kb, c0, LU, X, s_x); break;
+        default: rows_minus_block<T, NT, NB, 1>(n, lo, hi, k0, kb, c0, LU, X, s_x); break;
+        }
+        __syncthreads();
+        c0 += nc;
+    }
+}
+
 // Xt (n x nrhs, ld n) <- (L U)^{-1} Xt, one CTA, blocked by NB rows: each
 // diagonal block by cta_block_subst, then the rows still to solve take the
-// block's contribution (all threads).  s_blk: NB x NB of shared memory.
+// block's contribution (all threads).  s_blk: NB x NB of shared memory, s_x:
+// 8 NB more.
 template <typename T, int NT, int NB>
-__device__ void cta_lu_solve(int64_t n, int64_t nrhs, const T *LU, T *X, T *s_blk)
+__device__ void cta_lu_solve(int64_t n, int64_t nrhs, const T *LU, T *X, T *s_blk, T *s_x)
 {
     static_assert(NB <= 32, "one lane per row of a diagonal block");
-    const int tid = threadIdx.x;
     // forward, unit lower
     for (int64_t k0 = 0; k0 < n; k0 += NB) {
         const int kb = (int)(n - k0 < NB ? n - k0 : NB);
@@ -258,13 +324,7 @@ __device__ void cta_lu_solve(int64_t n, int64_t nrhs, const T *LU, T *X, T *s_bl
         __syncthreads();
         cta_block_subst<T, NT, true, true, false>(kb, nrhs, s_blk, X, n, k0);
         __syncthreads();
-        for (int64_t e = tid; e < (n - k0 - kb) * nrhs; e += NT) {
-            int64_t r = k0 + kb + e % (n - k0 - kb), c = e / (n - k0 - kb);
-            T s = T(0);
-            for (int p = 0; p < kb; p++) s = fma(LU[r + (k0 + p) * n], X[(k0 + p) + c * n], s);
-            X[r + c * n] -= s;
-        }
-        __syncthreads();
+        cta_minus_block<T, NT, NB>(n, nrhs, k0 + kb, n, k0, kb, LU, X, s_x);
     }
     // backward, upper
     const int64_t nblk = (n + NB - 1) / NB;
@@ -275,13 +335,7 @@ __device__ void cta_lu_solve(int64_t n, int64_t nrhs, const T *LU, T *X, T *s_bl
         __syncthreads();
         cta_block_subst<T, NT, false, false, false>(kb, nrhs, s_blk, X, n, k0);
         __syncthreads();
-        for (int64_t e = tid; e < k0 * nrhs; e += NT) {
-            int64_t r = e % k0, c = e / k0;
-            T s = T(0);
-            for (int p = 0; p < kb; p++) s = fma(LU[r + (k0 + p) * n], X[(k0 + p) + c * n], s);
-            X[r + c * n] -= s;
-        }
-        __syncthreads();
+        cta_minus_block<T, NT, NB>(n, nrhs, 0, k0, k0, kb, LU, X, s_x);
     }
 }
 
@@ -459,7 +513,7 @@ __device__ void solve_sys(const SysDesc &S, char *w, int d, int refine_max, doub
     cta_vec<NT>(n, d, U, 1, S.X, S.ldx, nrhs);
     for (int64_t e = tid; e < n * nrhs; e += NT) Xt[e] = narrow_to<T>(S.X[e % n + (e / n) * S.ldx]);
     __syncthreads();
-    cta_lu_solve<T, NT, NB>(n, nrhs, At, Xt, s_diag);
+    cta_lu_solve<T, NT, NB>(n, nrhs, At, Xt, s_diag, s_a);
     for (int64_t e = tid; e < n * nrhs; e += NT) S.X[e % n + (e / n) * S.ldx] = widen_of(Xt[e]);
     __syncthreads();
     cta_vec<NT>(n, d, V, 0, S.X, S.ldx, nrhs);
@@ -473,7 +527,7 @@ __device__ void solve_sys(const SysDesc &S, char *w, int d, int refine_max, doub
         cta_vec<NT>(n, d, U, 1, R, n, nrhs);
         for (int64_t e = tid; e < n * nrhs; e += NT) Xt[e] = narrow_to<T>(R[e]);
         __syncthreads();
-        cta_lu_solve<T, NT, NB>(n, nrhs, At, Xt, s_diag);
+        cta_lu_solve<T, NT, NB>(n, nrhs, At, Xt, s_diag, s_a);
         for (int64_t e = tid; e < n * nrhs; e += NT) R[e] = widen_of(Xt[e]);
         __syncthreads();
         cta_vec<NT>(n, d, V, 0, R, n, nrhs);
@@ -500,7 +554,7 @@ batched_kernel(const SysDesc *__restrict__ sys, const int *__restrict__ order, i
                rbt_batched_info *infos, char *work, int d, int refine_max, double tol, int fallback, int redo)
 {
     __shared__ int s_idx, s_flag;
-    __shared__ __align__(16) unsigned char smem_raw[sizeof(double) * (NB * NB + 2 * kTile * NB)];
+    __shared__ __align__(16) unsigned char smem_raw[sizeof(double) * kSmemElems<NB>];
     __shared__ double red[NT];
     __shared__ double s_anorm;
     const int tid = threadIdx.x;
