@@ -714,7 +714,8 @@ template <int S> static Slices carve(int64_t M, int64_t N, int64_t K, void *work
 }
 
 // The operands of one product C (M x N) -= A B and the balancing exponents of
-// its K (ka and ka2: of A's columns, the larger counts; kb: of B's rows).
+// its K (ka and ka2: of A's columns, the larger counts; kb: of B's rows, or
+// null to balance by A alone).
 template <int S> struct Operands {
     int64_t M, N;
     const elem_t<S> *A, *B;
@@ -776,10 +777,12 @@ static rbt_status products(int count, const Operands<S> *op, const Slices *sl, i
 }
 
 // A standalone update: its balancing exponents come from a pass of their own.
+// by_a: t_k = -E(A_.k), so that A's digits do not depend on B and a column of C
+// not on the other columns of B.
 template <int S>
 static rbt_status update(int64_t M, int64_t N, int64_t K, const elem_t<S> *A, int64_t lda, const elem_t<S> *B,
                          int64_t ldb, elem_t<S> *C, int64_t ldc, const int64_t *info, void *work, void *status,
-                         unsigned max_ctas, cudaStream_t stream, bool ta = false)
+                         unsigned max_ctas, cudaStream_t stream, bool ta = false, bool by_a = false)
 {
     rbt_status s = configure<S>();
     if (s != RBT_OK) return s;
@@ -789,11 +792,11 @@ static rbt_status update(int64_t M, int64_t N, int64_t K, const elem_t<S> *A, in
         // both exponent arrays start at kNoExp (every byte 0x80)
         RBT_CUDA_TRY(cudaMemsetAsync(sl.ka, 0x80, (size_t)rup(sl.Kp * 4, 256) * 2, stream));
         const int ca = (int)cdiv(M, 4096), na = ta ? (int)cdiv(M, 64) : ca * (int)K;
-        kexp_kernel<elem_t<S>><<<(unsigned)(na + cdiv(N, 64)), 256, 0, stream>>>((int)M, (int)K, (int)N, ca, na, ta, A,
+        kexp_kernel<elem_t<S>><<<(unsigned)(na + (by_a ? 0 : cdiv(N, 64))), 256, 0, stream>>>((int)M, (int)K, (int)N, ca, na, ta, A,
                                                                               lda, B, ldb, sl.ka, sl.kb);
         RBT_LAUNCH_CHECK();
     }
-    const Operands<S> op = {M, N, A, B, C, sl.ka, sl.ka, sl.kb, ta};
+    const Operands<S> op = {M, N, A, B, C, sl.ka, sl.ka, by_a ? nullptr : sl.kb, ta};
     return products<S, false>(1, &op, &sl, K, lda, ldb, ldc, info, status, max_ctas, stream);
 }
 
@@ -823,8 +826,11 @@ size_t oz_residual_workspace(int64_t n, int64_t nrhs)
 // R (n x nrhs) -= A X, or A^T X, in double by nine-digit sliced products over
 // pieces of 448 of the inner dimension: each reads A once, whatever the number
 // of right-hand sides, where the FP64 pipe takes n^2 nrhs multiply-adds at two
-// a clock and SM (3.4 ms for 32 at n = 8197).  *status (device, cleared by the
-// caller) becomes nonzero when a device wait gave up.
+// a clock and SM.  Balanced by A alone: an entry of the result is off by at most
+// 2^-57 K max_k |A_ik| 2^-E_k max_k 2^E_k |X_kj| a piece, whatever the other
+// columns of X hold (balanced against all of X, an isolated entry 2^40 in one
+// column left the others' residuals 20 bits short).  *status (device, cleared
+// by the caller) becomes nonzero when a device wait gave up.
 rbt_status oz_residual(int64_t n, int64_t nrhs, const double *A, int64_t lda, bool trans, const double *X, int64_t ldx,
                        double *R, int64_t ldr, const int64_t *info, void *work, int *status, cudaStream_t stream)
 {
@@ -832,7 +838,7 @@ rbt_status oz_residual(int64_t n, int64_t nrhs, const double *A, int64_t lda, bo
     for (int64_t k = 0; k < n; k += KMAX<9>) {
         const int64_t K = std::min<int64_t>(n - k, KMAX<9>);
         const rbt_status s = update<9>(n, nrhs, K, trans ? A + k : A + k * lda, lda, X + k, ldx, R, ldr, info, work, status,
-                                       (unsigned)device_sm_count(), stream, trans);
+                                       (unsigned)device_sm_count(), stream, trans, true);
         if (s != RBT_OK) return s;
     }
     return RBT_OK;

@@ -219,7 +219,7 @@ __device__ __forceinline__ int kshift(int a, int b)
 // for A (or its transpose stored K x M) and -1 for B.  Slice p goes to rows p rows_p ..
 // of a K-major [S rows_p][Kp] bf16 array (zeros past rows and K), the row
 // exponents to exps.  The balancing exponents of A's columns are the larger
-// of ka and ka2, those of B's rows kb.
+// of ka and ka2, those of B's rows kb; without kb the balancing is A's alone.
 template <typename TE> struct SliceJob {
     const TE *src;
     int64_t ld;
@@ -278,7 +278,10 @@ __global__ void __launch_bounds__(256) slice_kernel(const __grid_constant__ Slic
     const int rows = J.rows;
     const int64_t slice = (int64_t)J.rows_p * Kp;
     auto shifts = [&]() {  // t_k of every k
-        for (int k = tid; k < Kp; k += 256) ts[k] = k < K ? kshift(max(J.ka[k], J.ka2[k]), J.kb[k]) : 0;
+        for (int k = tid; k < Kp; k += 256) {
+            const int a = k < K ? max(J.ka[k], J.ka2[k]) : kNoExp;
+            ts[k] = a == kNoExp ? 0 : J.kb ? kshift(a, J.kb[k]) : -a;
+        }
     };
     if (J.by_rows) {
         const int ld_t = Kp + 2, r = tid % kSliceRows, kl = tid / kSliceRows;
