@@ -64,8 +64,9 @@ typedef enum {
                       n >= 768 runs the factorization's updates by exact digit
                       slicing on the BF16 tensor cores (nine 7-bit digits, 63
                       bits relative to each row's and column's largest entry)
-                      when A~ is dense enough for that to be no less accurate
-                      than double multiply-adds */
+                      when the entries of A~ are of like size up to row and
+                      column scalings, where that is no less accurate than
+                      double multiply-adds; else on the FP64 pipe */
     RBT_F32 = 1,   /* float storage, float SIMT trailing updates */
     RBT_TF32 = 2,  /* float storage, TF32 tensor-core trailing updates (fp32 accumulate) */
     RBT_BF16 = 3,  /* float storage, BF16 tensor-core operands (fp32 accumulate) */
