@@ -796,12 +796,14 @@ static rbt_status transform2_df64math(int64_t n, int d, const double *U, const d
 template <int L, typename TO>
 static void launch_fused2(int64_t n, int64_t h, int64_t ngroups, int k_hi, int pre_lo, int pre_hi,
                           const double *U, const double *V, int64_t ldw, const double *Ain,
-                          int64_t lda_in, TO *Aout, int64_t lda_out, cudaStream_t stream, bool rot)
+                          int64_t lda_in, TO *Aout, int64_t lda_out, cudaStream_t stream, bool rot, bool layered)
 {
     if constexpr (std::is_same<TO, double>::value && L <= 2) {
         // below n = 2048 too few CTAs of 16 column groups are left to fill the
-        // chip (n = 1003: 157 us against 32 us in the FP64 form; 4001: 232 / 298)
-        if (!rot && pre_hi < pre_lo && n >= 2048) {
+        // chip (n = 1003: 157 us against 32 us in the FP64 form; 2048: 61 / 107;
+        // 4001: 232 / 298).  The layer-by-layer form, what the fused one is
+        // compared with, stays in FP64.
+        if (!rot && !layered && pre_hi < pre_lo && n >= 2048) {
             const dim3 grid((unsigned)cdiv(ngroups, kTX), (unsigned)cdiv(ngroups, kFixGroups));
             fused2_fix_kernel<L><<<grid, kTX, 0, stream>>>(n, h, ngroups, k_hi, U, V, ldw, Ain, lda_in, Aout, lda_out);
             return;
@@ -850,9 +852,9 @@ static rbt_status transform2(int64_t n, int d, const double *U, const double *V,
         if (!last && sizeof(TO) != sizeof(double)) return RBT_ERR_UNSUPPORTED;
         TO *dst = Aout;
         switch (L) {
-        case 1: launch_fused2<1, TO>(n, h, ngroups, k_hi, pre_lo, pre_hi, U, V, ldw, src, ld_src, dst, lda_out, stream, rot); break;
-        case 2: launch_fused2<2, TO>(n, h, ngroups, k_hi, pre_lo, pre_hi, U, V, ldw, src, ld_src, dst, lda_out, stream, rot); break;
-        default: launch_fused2<3, TO>(n, h, ngroups, k_hi, pre_lo, pre_hi, U, V, ldw, src, ld_src, dst, lda_out, stream, rot); break;
+        case 1: launch_fused2<1, TO>(n, h, ngroups, k_hi, pre_lo, pre_hi, U, V, ldw, src, ld_src, dst, lda_out, stream, rot, max_l == 1); break;
+        case 2: launch_fused2<2, TO>(n, h, ngroups, k_hi, pre_lo, pre_hi, U, V, ldw, src, ld_src, dst, lda_out, stream, rot, max_l == 1); break;
+        default: launch_fused2<3, TO>(n, h, ngroups, k_hi, pre_lo, pre_hi, U, V, ldw, src, ld_src, dst, lda_out, stream, rot, max_l == 1); break;
         }
         RBT_LAUNCH_CHECK();
         src = reinterpret_cast<const double *>(Aout);
