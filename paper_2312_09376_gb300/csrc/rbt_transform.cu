@@ -231,7 +231,7 @@ fused2_kernel(int64_t n, int64_t h, int64_t ngroups, int k_hi, int pre_lo, int p
 // sum over the group, so an error of a few units (2^-58 of the group's largest
 // entry each) is below the half unit of double rounding of |U|^T |A| |V|, and
 // the FP64 form's roundings at every step are gone.  Measured at n = 16385, d =
-// 2: 4.46 -> 1.65 ms (965 -> 2600 GB/s), relative error in the 2-norm 2.3e-16
+// 2: 4.46 -> 1.70 ms (965 -> 2530 GB/s), relative error in the 2-norm 2.3e-16
 // -> 2.0e-16; what bounds it now is the issue of some 80 integer instructions
 // an entry.
 //
@@ -243,18 +243,26 @@ fused2_kernel(int64_t n, int64_t h, int64_t ngroups, int k_hi, int pre_lo, int p
 constexpr int kFixBits = 58;
 constexpr int kFixGroups = 16;  // column groups per CTA (their factors in shared memory)
 
-struct Frac {  // f 2^62 as two 31-bit halves
-    int hi, lo;
+struct Frac {  // f 2^62 as two 31-bit halves, and where a product's middle sum starts
+    int hi, lo, mid;
 };
 __device__ __forceinline__ Frac frac_of(double f)
 {
     const long long v = (long long)(f * 0x1p62);
-    return Frac{(int)(v >> 31), (int)(v & 0x7FFFFFFF)};
+    const int lo = (int)(v & 0x7FFFFFFF);
+    return Frac{(int)(v >> 31), lo, (1 << 30) + (lo >> 1)};
 }
+// The dropped vl f.lo (below one unit) is lo / 2 units of the middle sum in the
+// mean over vl, and the shift rounds down by half a unit of the result: mid
+// makes up for both, so that a product is off by no more than a unit and by
+// nothing in the mean.  (Without it every output lies 1.3 units low, those of
+// the sums alone 3.9, and an error common to all entries grows with n in the
+// operator norm, where rounding grows with its root.  Emulated at n = 2048, d =
+// 2, Gaussian: 5.2e-16 of ||A~||, with mid 4.8e-17, the FP64 form 1.4e-16.)
 __device__ __forceinline__ long long mul_frac(long long v, Frac f)
 {
     const int vh = (int)(v >> 31), vl = (int)(v & 0x7FFFFFFF);
-    const long long m = (long long)vh * f.lo + (long long)vl * f.hi;  // the dropped vl f.lo is below one unit
+    const long long m = (long long)vh * f.lo + ((long long)vl * f.hi + f.mid);
     return (long long)vh * f.hi + (m >> 31);
 }
 // the significand at 2^-58 of the binade of exponent field emax
