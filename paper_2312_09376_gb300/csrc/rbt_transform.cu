@@ -231,16 +231,21 @@ fused2_kernel(int64_t n, int64_t h, int64_t ngroups, int k_hi, int pre_lo, int p
 // sum over the group, so an error of a few units (2^-58 of the group's largest
 // entry each) is below the half unit of double rounding of |U|^T |A| |V|, and
 // the FP64 form's roundings at every step are gone.  Measured at n = 16385, d =
-// 2: 4.46 -> 1.70 ms (965 -> 2530 GB/s), relative error in the 2-norm 2.3e-16
+// 2: 4.46 -> 1.71 ms (965 -> 2510 GB/s), relative error in the 2-norm 2.3e-16
 // -> 2.0e-16; what bounds it now is the issue of some 80 integer instructions
 // an entry.
 //
 // A group with rows or columns past the matrix (nu rows pass through without
 // being summed), a factor outside (1/4, 6/5), an entry that is not finite, or a
 // largest entry near the ends of the exponent range takes the FP64 form.
+// So does one with entries more than 2^20 apart: where the large ones cancel
+// exactly (a column of one large value), the FP64 form keeps the small ones to
+// their last bit and the common fixed point would drop them, at 2^58 all of them.
+// (Of Gaussian groups 3 in 10^5.)
 // 64-bit: |v| < 2^58 grows by at most 4 in the butterflies and by
 // 4 (6/5)^2 / 2 < 2^1.6 over a layer: below 2^62 with two layers.
 constexpr int kFixBits = 58;
+constexpr unsigned kFixRange = 20;
 constexpr int kFixGroups = 16;  // column groups per CTA (their factors in shared memory)
 
 struct Frac {  // f 2^62 as two 31-bit halves, and where a product's middle sum starts
@@ -343,11 +348,16 @@ fused2_fix_kernel(int64_t n, int64_t h, int64_t ngroups, int k_hi, const double 
                 for (int s = 0; s < G; s++) {
                     x[s][t] = Ain[row0 + s * h + (col0 + t * h) * lda_in];
                 }
+            unsigned emin = ~0u;  // of the entries that are not zero, less one
 #pragma unroll
             for (int t = 0; t < G; t++)
 #pragma unroll
-                for (int s = 0; s < G; s++) emax = max(emax, (__double2hiint(x[s][t]) >> 20) & 0x7FF);
-            if (emax >= 100 && emax <= 2000) {
+                for (int s = 0; s < G; s++) {
+                    const int e = (__double2hiint(x[s][t]) >> 20) & 0x7FF;
+                    emax = max(emax, e);
+                    emin = min(emin, (unsigned)e - 1u);
+                }
+            if (emax >= 100 && emax <= 2000 && emin + 1u + kFixRange >= (unsigned)emax) {
                 long long v[G][G];
 #pragma unroll
                 for (int t = 0; t < G; t++)
