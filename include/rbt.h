@@ -315,7 +315,8 @@ rbt_status genp_update(int32_t prec, int64_t M, int64_t N, int64_t K, const floa
  * per prec).  B: double, n x nrhs, ldb.  For float factors the solve runs in
  * float (B rounded as it is read, the result widened back into B); for
  * double-float factors (RBT_DF64, RBT_DF64TC, RBT_DF64TC7) likewise in
- * double-float arithmetic.  work: genp_solve_workspace bytes.  The first int of `work` is cleared on
+ * double-float arithmetic.  work: genp_solve_workspace bytes, aligned to the
+ * element type of LU.  The first int of `work` is cleared on
  * entry and is nonzero after a call whose chained triangular solve gave up
  * waiting (B is then undefined; see rbt_debug_wait_limit).
  */
@@ -394,7 +395,8 @@ rbt_status rbt_norm_inf(int64_t n, const double *A, int64_t lda, double *d_out, 
  * Sec. 5); for RBT_DF64TC7 the first refactorization uses eight digits
  * (RBT_DF64TC) and only a stall of that one goes on to double.
  * A (n x n, lda) and B (n x nrhs, ldb) are not modified; X (n x nrhs, ldx)
- * receives the solution.  work: rbt_solve_workspace(opts, n, nrhs) bytes.
+ * receives the solution.  work: rbt_solve_workspace(opts, n, nrhs) bytes,
+ * aligned to 8 bytes (16 for the sliced precisions).
  * info (host) is written before return.  Returns RBT_OK, RBT_ZERO_PIVOT,
  * RBT_NONFINITE, RBT_NOT_CONVERGED or an error (RBT_ERR_TIMEOUT when any
  * bounded device wait of the call gave up).

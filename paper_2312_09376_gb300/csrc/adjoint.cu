@@ -224,8 +224,8 @@ rbt_status rbt_solve_adjoint(const rbt_opts *opts, const rbt_info *fwd, int64_t 
     };
     // many right-hand sides: residuals by sliced products, as in rbt_solve
     // (the first one's ||A^T|| from one column's pass)
-    void *fac = w + L.fac;
-    const size_t fac_bytes = L.sol - L.fac;
+    void *fac;
+    const size_t fac_bytes = factor_scratch(L, w, &fac);
     bool sliced_res = false;
     rbt_status st = sliced_residual(n, nrhs, A, lda, fac, fac_bytes, &sliced_res, s);
     if (st != RBT_OK) return st;

@@ -170,7 +170,7 @@ void solve_layout(const rbt_opts *o, int64_t n, int64_t nrhs, SolveLayout *out)
     size_t fac_ws = genp_factor_workspace_impl(n, o->prec, o->nb);
     if ((o->prec == RBT_F64 && o->nb == 0) || (o->prec != RBT_F64 && o->fallback))
         fac_ws = std::max(fac_ws, workspace64(n));
-    L.fac = take(fac_ws);
+    L.fac = take(fac_ws > 0 ? fac_ws + 16 : 0);  // its use starts on a 16-byte boundary (factor_scratch)
     L.sol = take(genp_solve_workspace(n, nr, RBT_F64));  // 8-byte entries: covers every precision and the GMRES form
     if (o->refine_mode == RBT_REFINE_GMRES) {
         // basis Q (m + 1 columns), z, w, a zero vector, dot-product partials, h / y
@@ -453,9 +453,9 @@ rbt_status rbt_solve(const rbt_opts *opts, int64_t n, int64_t nrhs, const double
     int64_t *d_info = (int64_t *)(w + L.info);
     double *scal = (double *)(w + L.scal);  // [0] ||A||, [1] berr
     double *res = (double *)(w + L.res);
-    void *fac = w + L.fac;
+    void *fac;
+    const size_t fac_bytes = factor_scratch(L, w, &fac);
     void *sol = w + L.sol;
-    size_t fac_bytes = L.sol - L.fac;
     const int64_t ldt = L.ldt;
     rbt_status st;
 

@@ -53,6 +53,15 @@ struct SolveLayout {
     int64_t ldt;
 };
 void solve_layout(const rbt_opts *o, int64_t n, int64_t nrhs, SolveLayout *out);
+// The factorization's scratch in a workspace at w, which may be aligned to a
+// double only, and its bytes: from a 16-byte boundary, as the tensor maps of the
+// sliced products want.
+inline size_t factor_scratch(const SolveLayout &L, char *w, void **fac)
+{
+    char *p = (char *)(((uintptr_t)(w + L.fac) + 15) / 16 * 16);
+    *fac = p;
+    return p < w + L.sol ? (size_t)(w + L.sol - p) : 0;
+}
 
 // The working-copy and one-sided transforms with the reference size's tile
 // alignment (align = n_b of Sec. 3's tiled rule; 0 or 1 = non-tiled) and the

@@ -498,6 +498,10 @@ static ChainScratch carve_chain(int64_t n, int64_t nrhs, size_t es, void *scratc
     s.nblk = cdiv(n > 0 ? n : 1, kTrsvNB);
     s.npad = s.nblk * kTrsvNB;
     s.err = (int *)w;
+    // published values are read two at a time, 16 bytes: the rest starts on such
+    // a boundary wherever the caller's buffer does (at most 12 bytes on, out of
+    // the 256 that chain_scratch_bytes adds)
+    w = (char *)(((uintptr_t)w + 15) / 16 * 16);
     s.counter = (unsigned *)(w + 256);
     s.xpub = w + 512;
     s.ones_bytes = 256 + 2 * (size_t)s.npad * (size_t)(nrhs > 0 ? nrhs : 1) * es;
