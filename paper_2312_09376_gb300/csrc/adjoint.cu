@@ -259,6 +259,7 @@ rbt_status rbt_solve_adjoint(const rbt_opts *opts, const rbt_info *fwd, int64_t 
     double berr = 0.0;
     RBT_CUDA_TRY(cudaMemcpyAsync(&berr, scal + 3, 8, cudaMemcpyDeviceToHost, s));
     RBT_CUDA_TRY(cudaStreamSynchronize(s));
+    if (h_res) return RBT_ERR_TIMEOUT;
     info->berr_unrefined = berr;
     int it = 0;
     while (!(berr <= opts->tol) && it < opts->refine_max) {
@@ -271,13 +272,14 @@ rbt_status rbt_solve_adjoint(const rbt_opts *opts, const rbt_info *fwd, int64_t 
         double prev = berr;
         RBT_CUDA_TRY(cudaMemcpyAsync(&berr, scal + 3, 8, cudaMemcpyDeviceToHost, s));
         RBT_CUDA_TRY(cudaStreamSynchronize(s));
+        if (h_res) return RBT_ERR_TIMEOUT;
         it++;
         if (!(berr < 0.9 * prev)) break;
     }
     bool to = false;
     st = timed_out(&to);
     if (st != RBT_OK) return st;
-    if (to || h_res) return RBT_ERR_TIMEOUT;
+    if (to) return RBT_ERR_TIMEOUT;
     info->iters = it;
     info->berr = berr;
     info->status = berr <= opts->tol ? RBT_OK : RBT_NOT_CONVERGED;
