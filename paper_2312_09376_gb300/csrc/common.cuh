@@ -36,17 +36,23 @@ enum ProfClass { kProfUpdate = 0, kProfTransform = 1, kProfPanel = 2, kProfSolve
 bool prof_on();
 void prof_record(int cls, cudaStream_t s, bool begin);
 
+// The outermost scope of a thread counts: what runs inside another class's (a
+// sliced residual's products) belongs to that one.
+inline thread_local int prof_depth = 0;
+
 struct ProfScope {
     int cls;
     cudaStream_t s;
     bool on;
-    ProfScope(int c, cudaStream_t st) : cls(c), s(st), on(prof_on())
+    ProfScope(int c, cudaStream_t st) : cls(c), s(st), on(prof_on() && prof_depth == 0)
     {
+        prof_depth++;
         if (on) prof_record(cls, s, true);
     }
     ~ProfScope()
     {
         if (on) prof_record(cls, s, false);
+        prof_depth--;
     }
 };
 
