@@ -156,6 +156,13 @@ class Clocks:
                 "reasons": sorted(reasons), "samples": len(rows)}
 
 
+def timing_record(each, clocks):
+    """Record of timed calls (milliseconds each).  Its size does not grow with their
+    number: the whole report is one line, which a reader may take in part only."""
+    return {"reps": len(each), "mean_ms": statistics.fmean(each), "min_ms": min(each), "max_ms": max(each),
+            "ci99_ms": ci99(each), "clocks": clocks}
+
+
 def timed(fn, reps, warmup, index, stream=None, min_ms=0.0):
     """Time `fn` on the device: `warmup` untimed calls, then at least `reps`
     timed calls (more while the timed calls sum to less than min_ms), one
@@ -179,9 +186,7 @@ def timed(fn, reps, warmup, index, stream=None, min_ms=0.0):
         marks.append(e)
     torch.cuda.synchronize()
     clk = clocks.stop()
-    each = [marks[i].elapsed_time(marks[i + 1]) for i in range(len(outs))]
-    return {"reps": len(each), "mean_ms": statistics.fmean(each), "ci99_ms": ci99(each), "each_ms": each,
-            "clocks": clk}, outs
+    return timing_record([marks[i].elapsed_time(marks[i + 1]) for i in range(len(outs))], clk), outs
 
 
 def _cpulist(text):
@@ -603,14 +608,14 @@ def run_ours(args):
                                                                         if prec == "df64tc7" else "FP64 refactor"),
                    "l2": "inputs 12.8 GB >> L2, no flush",
                    "parallelism": "replicas" if world > 1 else "single", "kind": args.kind, "align": args.align},
-        "step_ms": {"each": step_ms, "ci99": ci99(step_ms)},
-        "berr": max(i["berr"] for i in timed_infos), "iters": [i["iters"] for i in timed_infos],
-        "fell_back": [i["fell_back"] for i in timed_infos],
+        "step_ms": {"min": min(step_ms), "max": max(step_ms), "ci99": ci99(step_ms)},
+        "berr": max(i["berr"] for i in timed_infos), "iters": sorted({i["iters"] for i in timed_infos}),
+        "fell_back": sorted({i["fell_back"] for i in timed_infos}),
         "roofline": roof, "transform": transform, "transform_f32_pass": f32_pass,
         "breakdown_ms_per_step": {k: v[0] / args.steps for k, v in prof.items()},
         "e2e": {"value": replicas.aggregate_tflops(world, flops(n), ms_e2e), "unit": "TFLOP/s",
                 "h2d_bytes_per_step": 8 * n * n + 8 * n, "d2h_bytes_per_step": 8 * n, "ms_per_step": ms_e2e,
-                "each_ms": e2e_each, "api": "rbt_solve_host (pinned host A, b, x)",
+                "min_ms": min(e2e_each), "max_ms": max(e2e_each), "api": "rbt_solve_host (pinned host A, b, x)",
                 "same_x_as_device_run": e2e_same, "copy_engine_h2d_gbs": ce_gbs, "host_numa_node": node,
                 "copy_overhead_ms": ms_e2e - ms},
         "gpu_launches": launches,
