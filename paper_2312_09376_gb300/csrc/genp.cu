@@ -886,6 +886,24 @@ template rbt_status gemm_sub_simt<df64>(int64_t, int64_t, int, const df64 *, int
 
 // ------------------------------------------------------------ factor driver
 
+// Which kernels take a step of kb columns, nb but in the last one.  The 64-column
+// ones up to 64 (the only ones that deliver kmax), but a
+// narrow step in double or float fills a quarter or half of diag64_kernel's panels
+// and a few of trsm64_kernel's lanes.  Milliseconds of a factorization, both older
+// kernels / older diagonal factor only / both 64-column ones:
+//   double n = 1003  nb 16: 3.29 / 3.22 / 3.60    nb 32: 3.07 / 2.87 / 3.38
+//          n = 2500  nb 16: 15.49 / 15.78 / 16.75  nb 32: 14.81 / 14.76 / 16.04
+//   float  n = 1003  nb 16: 2.29 / 2.16 / 2.29    nb 32: 1.60 / 1.41 / 1.54
+// (double-float: the 64-column ones throughout.)
+template <typename T> static bool use_diag64(int kb, int nb, const int *kmax)
+{
+    return kb <= kP && (kmax || nb > 32 || std::is_same<T, df64>::value);
+}
+template <typename T> static bool use_trsm64(int kb, int nb, const int *kmax)
+{
+    return kb <= kP && (kmax || nb > 16 || !std::is_same<T, double>::value);
+}
+
 template <typename T>
 rbt_status genp_panel_steps(int64_t n, T *A, int64_t lda, int64_t *info, int nb, int64_t k0, int64_t k_end,
                             bool trailing_simt, cudaStream_t stream, int64_t panel_end, int *kmax)
@@ -895,7 +913,7 @@ rbt_status genp_panel_steps(int64_t n, T *A, int64_t lda, int64_t *info, int nb,
         int64_t rest = n - k - kb;
         {
             ProfScope ps(kProfPanel, stream);
-            if (kb <= kP) {
+            if (use_diag64<T>(kb, nb, kmax)) {
                 diag64_kernel<T><<<1, 256, 0, stream>>>(k, kb, A, lda, info);
             } else {
                 size_t sm = (size_t)kb * kb * sizeof(T);
@@ -903,7 +921,7 @@ rbt_status genp_panel_steps(int64_t n, T *A, int64_t lda, int64_t *info, int nb,
             }
             RBT_LAUNCH_CHECK();
             if (rest <= 0) continue;
-            if (kb <= kP) {
+            if (use_trsm64<T>(kb, nb, kmax)) {
                 if constexpr (std::is_same<T, double>::value)
                     launch_trsm64<T, 8, 16, 1>(k, kb, n, A, lda, info, panel_end, kmax, stream);
                 else if (2 * cdiv(rest, 64) >= kNumSMs)
