@@ -265,13 +265,14 @@ __device__ __forceinline__ void cta_load_block(int kb, const T *LU, int64_t n, i
     for (int e = threadIdx.x; e < kb * kb; e += NT) s_blk[e] = LU[(k0 + e % kb) + (k0 + e / kb) * n];
 }
 
-// Rows [lo, hi) of X(:, c0 .. c0 + NC) -= LU(:, k0 .. k0 + kb) times the
+// Rows [lo, hi) of X(:, c0 .. c0 + 8) -= LU(:, k0 .. k0 + kb) times the
 // block's solved rows (in s_x): one row per thread, its entries of LU read
-// once for NC right-hand sides.
-template <typename T, int NT, int NB, int NC>
+// once for the eight right-hand sides.
+template <typename T, int NT, int NB>
 __device__ __forceinline__ void rows_minus_block(int64_t n, int64_t lo, int64_t hi, int64_t k0, int kb, int64_t c0,
                                                  const T *LU, T *X, const T *s_x)
 {
+    constexpr int NC = kMaxRhsChunk;
     for (int64_t r = lo + threadIdx.x; r < hi; r += NT) {
         T s[NC];
 #pragma unroll
@@ -287,42 +288,36 @@ __device__ __forceinline__ void rows_minus_block(int64_t n, int64_t lo, int64_t 
     }
 }
 
-// The same for every right-hand side, in chunks of 8, 4, 2 and 1 (s_x: 8 NB
-// elements of shared memory).  Small systems have too few rows for that, and
-// the wider types' sums for eight columns spill: there a thread takes one row
-// of one right-hand side (same sums, bit for bit).  400 systems of order 60 ..
-// 400 with up to 8 columns: float 13.9 -> 12.8 ms, double 18.3 -> 18.9 ms with
-// the chunks; 64 systems of order 16 .. 90: no rows to spare.
+// The same for every right-hand side.  In float and from order 384 by eights
+// (s_x: 8 NB elements of shared memory); the rest, the wider types (whose sums
+// for eight columns spill) and smaller systems (too few rows) take one row of one
+// right-hand side a thread (same sums, bit for bit).  Milliseconds, float, 152
+// systems, by eights (by fours, twos and one for fewer) / an entry a thread:
+// order 384 .. 420, 1 / 3 / 5 / 8 columns 11.3 / 10.8, 11.9 / 11.3, 13.0 / 12.3,
+// 16.7 / 17.3; order 600 .. 700, 1 / 3 / 8 columns 31.7 / 30.6, 48.6 / 46.1, 45.2
+// / 45.9.
 constexpr int64_t kRowsPerThreadMin = 384;
 template <typename T, int NT, int NB>
 __device__ __forceinline__ void cta_minus_block(int64_t n, int64_t nrhs, int64_t lo, int64_t hi, int64_t k0, int kb,
                                                 const T *LU, T *X, T *s_x)
 {
-    if (sizeof(T) > 4 || n < kRowsPerThreadMin) {
-        const int64_t rows = hi - lo;
-        for (int64_t e = threadIdx.x; e < rows * nrhs; e += NT) {
-            const int64_t r = lo + e % rows, c = e / rows;
-            T s = T(0);
-            for (int p = 0; p < kb; p++) s = fma(LU[r + (k0 + p) * n], X[(k0 + p) + c * n], s);
-            X[r + c * n] -= s;
+    constexpr int NC = kMaxRhsChunk;
+    int64_t c0 = 0;
+    if (sizeof(T) == 4 && n >= kRowsPerThreadMin)
+        for (; c0 + NC <= nrhs; c0 += NC) {
+            for (int e = threadIdx.x; e < kb * NC; e += NT) s_x[e / kb * NB + e % kb] = X[(k0 + e % kb) + (c0 + e / kb) * n];
+            __syncthreads();
+            rows_minus_block<T, NT, NB>(n, lo, hi, k0, kb, c0, LU, X, s_x);
+            __syncthreads();
         }
-        __syncthreads();
-        return;
+    const int64_t rows = hi - lo;
+    for (int64_t e = threadIdx.x; e < rows * (nrhs - c0); e += NT) {
+        const int64_t r = lo + e % rows, c = c0 + e / rows;
+        T s = T(0);
+        for (int p = 0; p < kb; p++) s = fma(LU[r + (k0 + p) * n], X[(k0 + p) + c * n], s);
+        X[r + c * n] -= s;
     }
-    for (int64_t c0 = 0; c0 < nrhs;) {
-        const int64_t left = nrhs - c0;
-        const int nc = left >= 8 ? 8 : left >= 4 ? 4 : left >= 2 ? 2 : 1;
-        for (int e = threadIdx.x; e < kb * nc; e += NT) s_x[e / kb * NB + e % kb] = X[(k0 + e % kb) + (c0 + e / kb) * n];
-        __syncthreads();
-        switch (nc) {
-        case 8: rows_minus_block<T, NT, NB, 8>(n, lo, hi, k0, kb, c0, LU, X, s_x); break;
-        case 4: rows_minus_block<T, NT, NB, 4>(n, lo, hi, k0, kb, c0, LU, X, s_x); break;
-        case 2: rows_minus_block<T, NT, NB, 2>(n, lo, hi, k0, kb, c0, LU, X, s_x); break;
-        default: rows_minus_block<T, NT, NB, 1>(n, lo, hi, k0, kb, c0, LU, X, s_x); break;
-        }
-        __syncthreads();
-        c0 += nc;
-    }
+    __syncthreads();
 }
 
 // Xt (n x nrhs, ld n) <- (L U)^{-1} Xt, one CTA, blocked by NB rows: each
