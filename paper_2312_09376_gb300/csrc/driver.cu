@@ -235,8 +235,11 @@ rbt_status factor_copy(int64_t n, int prec, void *At, int64_t ldt, int64_t *d_in
 
 namespace rbt {
 
-// Fewest right-hand sides for sliced residuals: at n = 8197 the FP64 pipe takes
-// 0.14 ms a right-hand side (4.5 ms for 32), the sliced form 2.1 ms for up to 48.
+// Fewest right-hand sides for sliced residuals, from the order of the sliced
+// updates on.  One residual of 32 at n = 8197: 6.2 ms on the FP64 pipe, 2.0 ms
+// sliced.  Whole double solves with 15 (FP64 pipe) and 16 (sliced) right-hand
+// sides, two residuals each: n = 768 3.52 / 2.55 ms, 1003 4.59 / 3.28, 1500 6.02 /
+// 4.78.
 constexpr int64_t kSlicedResRhs = 16;
 
 rbt_status sliced_residual(int64_t n, int64_t nrhs, const double *A, int64_t lda, void *scratch, size_t bytes, bool *yes,

@@ -40,7 +40,7 @@
 // like size; a sparse matrix's fill-in can be smaller than its row's maximum
 // by more than the ten spare bits, so rbt_solve asks first (spread.cu).  The
 // FP64 pipe's 1.2 TFLOP/s bounded such factorizations: update class at n =
-// 8197 307 ms, now 15.7 ms and 9.5 ms of slicing.
+// 8197 307 ms, now 14.3 ms and 1.6 ms of slicing.
 //
 // Kernel: persistent, one CTA per SM, 128 x 64 output tiles (S accumulators
 // x 64 columns in the 512 TMEM columns) dealt round-robin in an L2-friendly

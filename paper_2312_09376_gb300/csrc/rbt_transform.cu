@@ -232,8 +232,8 @@ fused2_kernel(int64_t n, int64_t h, int64_t ngroups, int k_hi, int pre_lo, int p
 // entry each) is below the half unit of double rounding of |U|^T |A| |V|, and
 // the FP64 form's roundings at every step are gone.  Measured at n = 16385, d =
 // 2: 4.46 -> 1.71 ms (965 -> 2510 GB/s), relative error in the 2-norm 2.3e-16
-// -> 2.0e-16; what bounds it now is the issue of some 80 integer instructions
-// an entry.
+// -> 2.0e-16; what bounds it now is the issue of some 130 instructions an entry
+// (62% of the ALU pipe, at eleven warps an SM).
 //
 // A group with rows or columns past the matrix (nu rows pass through without
 // being summed), a factor outside (1/4, 6/5), an entry that is not finite, or a
@@ -818,8 +818,8 @@ static void launch_fused2(int64_t n, int64_t h, int64_t ngroups, int k_hi, int p
 {
     if constexpr (std::is_same<TO, double>::value && L <= 2) {
         // below n = 2048 too few CTAs of 16 column groups are left to fill the
-        // chip (n = 1003: 157 us against 32 us in the FP64 form; 2048: 61 / 107;
-        // 4001: 232 / 298).  The layer-by-layer form, what the fused one is
+        // chip (n = 1003: 157 us against 32 us in the FP64 form; 2048: 68 / 107;
+        // 4001: 262 / 315).  The layer-by-layer form, what the fused one is
         // compared with, stays in FP64.
         if (!rot && !layered && pre_hi < pre_lo && n >= 2048) {
             const dim3 grid((unsigned)cdiv(ngroups, kTX), (unsigned)cdiv(ngroups, kFixGroups));

@@ -551,6 +551,8 @@ static rbt_status launch_chain(int64_t n, int64_t nrhs, const TF *LU, int64_t ld
 //           n = 20001:  8 rhs 4512 / 4658;               16 rhs 7915 / 6429
 //   float   n = 8197:   4 rhs 418 / 459 / 644 (R = 4);   16 rhs 1017 / 658 / 692
 //           n = 4001:  32 rhs 417 / 290 / 352;           64 rhs 744 / 449 / 384
+//           n = 4001:  256 / 1024 rhs 1021 / 3421 at R = 4 (blocked sweep 30.7 / 118.8 ms;
+//                      pairs 3.7 / 14.2, sweep 99 / 386 ms)
 // In double the FP64 pipe is the bound either way (32 rhs at n = 8197: 4610 /
 // 5488): always one.  Pairs with R = 4 would spill.
 template <typename T, typename TF, bool TRANS>
